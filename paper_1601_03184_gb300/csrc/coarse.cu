@@ -10,6 +10,13 @@ namespace mrhs {
 namespace {
 
 constexpr int kSites = 8;  // sites staged per chunk in the contractions
+// Right-hand sides up to which the coarse stencil takes a warp per row
+// (k_apply_dc_rows). One thread per (eight rows, right-hand side) leaves the
+// GPU idle at few of them: 1 right-hand side, 512 aggregates, 2ntv = 40, FP32:
+// 397 -> 21 us per application; 4: 132 -> 36; 8: 119 -> 72 (the whole call; at
+// 4096 aggregates, 2ntv = 48: 890 -> 173, 675 -> 308, 760 -> 636 us). From 9 on
+// the row's registers would be read for a second group of vectors.
+constexpr int kRowsMaxRhs = 8;
 
 // One CTA per (aggregate A, stencil entry k). Columns (h', j), rows (h, i):
 //   k = 0:      sum_{x in A} P_(h,i)(x)^dag [A(x) + hops inside A] P_(h',j)
@@ -425,6 +432,89 @@ __global__ void k_apply_dc_tiled(const cx<typename Real<SC>::type>* __restrict__
   for (int a = 0; a < 8; ++a) st<SC, R>(y, (size_t)b * nc + row0 + a, N, r, acc[a]);
 }
 
+// Few right-hand sides (the V-cycle of a solve has one): CTA (b, g) takes rows
+// g, g + gridDim.y, ... eight warps wide of aggregate alist[b]; the x blocks of
+// the nine neighbours are staged once, one vector after the other, and a warp
+// holds a whole row of the nine blocks in registers (lane l: the CH columns at
+// CH l, then 32 CH further on, NP times; CH NP 32 >= nc), so that all of its
+// loads of D_c are in flight together and every one serves NB right-hand sides.
+template <class R, int CH>
+__device__ __forceinline__ void ld_cols(cx<R> v[CH], const cx<R>* p) {
+  if constexpr (CH == 2 && sizeof(R) == 4) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = mk<R>(t.x, t.y), v[1] = mk<R>(t.z, t.w);
+  } else {
+#pragma unroll
+    for (int i = 0; i < CH; ++i) v[i] = p[i];
+  }
+}
+template <class SC, int NB, int CH, int NP>
+__global__ void __launch_bounds__(256) k_apply_dc_rows(const cx<typename Real<SC>::type>* __restrict__ Dc,
+                                                       DcPartArgs<SC> pa, SC* __restrict__ y,
+                                                       const int* __restrict__ aggnbr, int nc, int N) {
+  using R = typename Real<SC>::type;
+  extern __shared__ double smem_d[];
+  cx<R>* sx = reinterpret_cast<cx<R>*>(smem_d);  // [N][9][nc]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = blockIdx.x;
+  const int A = pa.alist ? pa.alist[b] : b;
+  for (int k = pa.kb + warp; k < pa.ke; k += 8) {
+    int B = k == 0 ? A : aggnbr[A * 8 + k - 1];
+    if (pa.pos) B = pa.pos[B];
+    const SC* x = (k == 0 ? pa.x0 : pa.xh) + (size_t)B * nc * 2 * N;
+    for (int e = lane; e < nc * N; e += 32) {
+      const int r = e % N, col = e / N;
+      sx[(r * 9 + k) * nc + col] = ld<SC, R>(x, col, N, r);
+    }
+  }
+  const cx<R>* D = Dc + (size_t)A * 9 * nc * nc;
+  __syncthreads();
+  for (int row = blockIdx.y * 8 + warp; row < nc; row += gridDim.y * 8) {
+    cx<R> d[9][NP][CH];
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const int col = CH * (lane + 32 * p);
+        const bool on = k >= pa.kb && k < pa.ke && col < nc;
+#pragma unroll
+        for (int i = 0; i < CH; ++i) d[k][p][i] = mk<R>(0, 0);
+        if (on) ld_cols<R, CH>(d[k][p], D + ((size_t)k * nc + row) * nc + col);
+      }
+    cx<R> acc[NB];
+#pragma unroll
+    for (int e = 0; e < NB; ++e) {
+      acc[e] = mk<R>(0, 0);
+      if (e >= N) continue;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        if (k < pa.kb || k >= pa.ke) continue;
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+          const int col = CH * (lane + 32 * p);
+          if (col < nc) {
+#pragma unroll
+            for (int i = 0; i < CH; ++i) fma_(acc[e], d[k][p][i], sx[(e * 9 + k) * nc + col + i]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < NB; ++e)
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) {
+        acc[e].re += __shfl_xor_sync(0xffffffffu, acc[e].re, o);
+        acc[e].im += __shfl_xor_sync(0xffffffffu, acc[e].im, o);
+      }
+#pragma unroll
+    for (int e = 0; e < NB; ++e)
+      if (lane == e && e < N) {
+        const size_t out = (size_t)b * nc + row;
+        st<SC, R>(y, out, N, e, pa.add ? ld<SC, R>(pa.add, out, N, e) + acc[e] : acc[e]);
+      }
+  }
+}
+
 // u = P uc with one thread per (site, chirality, right-hand side): 6 outputs
 // share every load of uc
 template <class SP, class SC, class SU>
@@ -810,7 +900,16 @@ void apply_Dc_part(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, int dtype) 
     using SC = std::remove_pointer_t<decltype(tag)>;
     using R = typename Real<SC>::type;
     const DcPartArgs<SC> pa{pt.alist, pt.pos, pt.kb, pt.ke, (const SC*)pt.x0, (const SC*)pt.xh, (const SC*)pt.add};
-    if (nc % 8 == 0) {
+    const size_t smem_rows = sizeof(cx<R>) * 9 * (size_t)nc * nrhs;
+    if (nrhs <= kRowsMaxRhs && smem_rows <= 48 * 1024) {
+      auto pick = [&](auto one, auto two, auto four) { return nc <= 32 ? one : nc <= 64 ? two : four; };
+      auto kern = nrhs == 1   ? pick(k_apply_dc_rows<SC, 1, 1, 1>, k_apply_dc_rows<SC, 1, 2, 1>, k_apply_dc_rows<SC, 1, 2, 2>)
+                  : nrhs <= 4 ? pick(k_apply_dc_rows<SC, 4, 1, 1>, k_apply_dc_rows<SC, 4, 2, 1>, k_apply_dc_rows<SC, 4, 2, 2>)
+                              : pick(k_apply_dc_rows<SC, 8, 1, 1>, k_apply_dc_rows<SC, 8, 2, 1>, k_apply_dc_rows<SC, 8, 2, 2>);
+      const int per = nrhs <= 2 ? 1 : 2;  // rows per warp: the staged x is shared by more rows when it is larger
+      kern<<<dim3(pt.na, (nc + 8 * per - 1) / (8 * per)), 256, smem_rows, c->stream>>>((const cx<R>*)c->Dc, pa, (SC*)yc,
+                                                                                     c->aggnbr, nc, nrhs);
+    } else if (nc % 8 == 0) {
       const size_t work = (size_t)pt.na * (nc / 8) * nrhs;
       k_apply_dc_tiled<SC><<<grid_for(work, 128), 128, 0, c->stream>>>((const cx<R>*)c->Dc, pa, (SC*)yc, c->aggnbr,
                                                                         nc, nrhs, work);

@@ -1,0 +1,43 @@
+"""The coarse stencil of few right-hand sides (a warp per coarse row) at the
+edges of its range, against the oracle's stencil on the GPU's own D_c.
+
+Every output is a sum of 9 * 2ntv complex products: in any order of the sums
+the error of one entry is below gamma_n (|D_c| |x|) with n = 2 * 9 * 2ntv + 2
+real terms of unit roundoff u (and sqrt(2) for the two parts of an entry)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1601_03184_gb300 import (MRHS_F32, MRHS_F64, MRHS_PREC_FP32, MRHS_PREC_FP64, Lattice, inputs)
+
+pytestmark = pytest.mark.gpu
+
+DIMS, AGG = (4, 8, 4, 8), (2, 4, 2, 2)
+
+
+# 2ntv = 2, 10 and 32 (one column per lane), 34 and 64 (two), 66 and 72 (two, twice)
+# (D_c of an FP64 context is built up to ntv = 32)
+@pytest.mark.parametrize("ntv,prec", [(n, MRHS_PREC_FP32) for n in (1, 5, 16, 17, 32, 33, 36)]
+                         + [(n, MRHS_PREC_FP64) for n in (1, 5, 16, 17, 32)])
+def test_coarse_stencil_of_few_vectors(ntv, prec):
+    wd = MRHS_F32 if prec == MRHS_PREC_FP32 else MRHS_F64
+    u = 2.0 ** (-24 if prec == MRHS_PREC_FP32 else -53)
+    lat = Lattice(DIMS, AGG, ntv, prec)
+    lat.set_gauge(inputs.gauge_field(DIMS, 0.5, 1401))
+    lat.build_clover(-0.1, 1.2)
+    lat.set_tv(lat.to_device(inputs.test_vectors(ntv, DIMS, 2401), wd), wd)
+    lat.build_P()
+    lat.build_Dc()
+    Dc = lat.get_Dc()
+    n = 2 * 9 * 2 * ntv + 2
+    for nrhs in (1, 2, 3, 4, 5, 8, 9):
+        x = inputs.gaussian_field((nrhs, lat.nagg, 2 * ntv), 4401)
+        if wd == MRHS_F32:
+            x = x.astype(np.complex64).astype(np.complex128)
+        xd, yd = lat.to_device(x, wd, coarse=True), lat.field(nrhs, wd, coarse=True)
+        lat.apply_Dc(xd, yd, nrhs, wd)
+        ref = oracle.apply_Dc(DIMS, AGG, Dc, x)
+        size = oracle.apply_Dc(DIMS, AGG, np.abs(Dc).astype(np.complex128), np.abs(x).astype(np.complex128)).real
+        err = np.abs(lat.to_host(yd, nrhs, wd, coarse=True) - ref)
+        assert np.all(err <= 2 ** 0.5 * n * u / (1 - n * u) * size + 1e-300), nrhs
+    lat.close()
