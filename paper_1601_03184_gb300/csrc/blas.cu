@@ -7,7 +7,11 @@
 #include <algorithm>
 #include <cstdint>
 
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace mrhs {
 namespace {
@@ -23,137 +27,173 @@ int n_chunks(size_t rows, int N) {
 }
 
 // partial[k][chunk][r] = sum over the chunk's rows of conj(X_k) * Y, for the
-// group of up to kKG vectors k = kKG*blockIdx.y + j: every element of Y read
-// serves the whole group
-constexpr int kKG = 8;
+// group of up to KG vectors k = KG*blockIdx.y + j: every element of Y read
+// serves the whole group. A thread takes VEC right-hand sides of a row (VEC =
+// 4: FP32, N % 4 == 0, 16-byte loads), Q = N / VEC threads a row, and a warp
+// 32 / Q rows at a time (a row spans warps when Q > 32). Bound by the loads when
+// there are enough rows; at few rows (coarse fields) by the sums across the
+// threads, and there by FP64, which this GPU adds at 2 per clock and SM. So
+// threads of FP32 data with at most kMaxRows rows sum them in FP32, the rows
+// of a warp are joined by FP32 shuffles (a tree: five more roundings) and only
+// the warps' sums are FP64; otherwise (FLUSH) a thread adds its FP32 sums of
+// kFlush rows in FP64 and the threads are joined by a tree in FP64.
+// A chunk is one CTA, or a cluster of eight when the chunks alone would leave
+// most of the GPU idle: the ranks take eighths of the chunk and the first adds
+// their sums in order, so that the partials, and the workspace they need, stay
+// one per chunk.
+constexpr int kKG = 4;          // vectors per group (its sums: up to 40 KB of shared memory)
+constexpr int kFlush = 32;
+constexpr int kMaxRows = 128;
+constexpr int kClusterCtas = 8;
+// CTAs (two for each of the 152 SMs) below which a chunk becomes a cluster.
+// Measured per call: 1 vector of 4096 rows, FP32 (one CTA and a serial FP64 sum
+// before) 97 -> 23 us; 1 to 20 vectors of 16384 x 32 (32 to 160 CTAs) 35 -> 28 us,
+// and 37 -> 20 us at 12800 x 20.
+constexpr int kClusterBelow = 304;
 
-template <class S>
-__global__ void __launch_bounds__(kBlock) k_multi_dot(const S* X, size_t stride, int K, const S* Y, size_t rows, int N,
-                                                      int nchunk, double* part) {
-  using R = typename Real<S>::type;
-  __shared__ double sre[kBlock], sim[kBlock];
-  const int k0 = blockIdx.y * kKG, ch = blockIdx.x;
-  const int nk = min(kKG, K - k0);
-  const size_t r0 = rows * ch / nchunk, r1 = rows * (ch + 1) / nchunk;
-  const int lanes = blockDim.x / N;
-  const int tid = threadIdx.x, r = tid % N, lane = tid / N;
-  double are[kKG], aim[kKG];
-  R pre[kKG], pim[kKG];
-#pragma unroll
-  for (int j = 0; j < kKG; ++j) are[j] = aim[j] = 0, pre[j] = pim[j] = 0;
-  if (lane < lanes) {
-    int cnt = 0;
-    for (size_t row = r0 + lane; row < r1; row += lanes) {
-      const R yr = to_r(Y[fidx(row, 0, N, r)]), yi = to_r(Y[fidx(row, 1, N, r)]);
-#pragma unroll
-      for (int j = 0; j < kKG; ++j) {
-        if (j < nk) {
-          const S* Xk = X + (size_t)(k0 + j) * stride;
-          const R xr = to_r(Xk[fidx(row, 0, N, r)]), xi = to_r(Xk[fidx(row, 1, N, r)]);
-          pre[j] = fma(xr, yr, fma(xi, yi, pre[j]));
-          pim[j] = fma(xr, yi, fma(-xi, yr, pim[j]));
-        }
-      }
-      if (++cnt == 32) {
-#pragma unroll
-        for (int j = 0; j < kKG; ++j) are[j] += pre[j], aim[j] += pim[j], pre[j] = pim[j] = 0;
-        cnt = 0;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < kKG; ++j) are[j] += pre[j], aim[j] += pim[j];
-  }
-  for (int j = 0; j < nk; ++j) {
-    sre[tid] = are[j];
-    sim[tid] = aim[j];
-    __syncthreads();
-    if (tid < N) {
-      double a = 0, b = 0;
-      for (int l = 0; l < lanes; ++l) {
-        a += sre[l * N + tid];
-        b += sim[l * N + tid];
-      }
-      double* o = part + (((size_t)(k0 + j) * nchunk + ch) * N + tid) * 2;
-      o[0] = a;
-      o[1] = b;
-    }
-    __syncthreads();
+template <class S, int VEC>
+__device__ __forceinline__ void ld_row(const S* p, typename Real<S>::type v[VEC]) {
+  if constexpr (VEC == 4) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+  } else {
+    v[0] = to_r(p[0]);
   }
 }
 
-// The same for FP32 arrays with N % 4 == 0: a thread takes four right-hand
-// sides (16-byte loads of the real and the imaginary row) and sums its rows
-// of the chunk in FP32 before the CTA adds the threads' sums in FP64. Used
-// when a thread has at most kMaxRows4 rows of the chunk (the coarse fields).
-constexpr int kMaxRows4 = 128;
+// rows that one pass of a CTA covers
+__host__ __device__ __forceinline__ int dot_lanes(int Q) { return Q <= 32 ? (kBlock / 32) * (32 / Q) : kBlock / Q; }
 
-constexpr int kKG4 = 4;  // vectors per group (register budget of 16 FP32 sums each)
-
-__global__ void __launch_bounds__(kBlock, 2) k_multi_dot4(const float* __restrict__ X, size_t stride, int K,
-                                                          const float* __restrict__ Y, size_t rows, int N, int nchunk,
-                                                          double* __restrict__ part) {
-  constexpr int kKG = kKG4;
-  __shared__ double sre[4 * kBlock], sim[4 * kBlock];  // [lanes][N]
-  const int k0 = blockIdx.y * kKG, ch = blockIdx.x;
-  const int nk = min(kKG, K - k0);
-  const size_t r0 = rows * ch / nchunk, r1 = rows * (ch + 1) / nchunk;
-  const int Q = N / 4, lanes = kBlock / Q;
-  const int tid = threadIdx.x, q = tid % Q, lane = tid / Q;
-  float pre[kKG][4], pim[kKG][4];
+template <class S, int VEC, int KG, bool FLUSH>
+__global__ void __launch_bounds__(kBlock, 2) k_multi_dot(const S* __restrict__ X, size_t stride, int K,
+                                                         const S* __restrict__ Y, size_t rows, int N, int nchunk,
+                                                         int ranks, double* __restrict__ part) {
+  using R = typename Real<S>::type;
+  // FLUSH: [KG][lanes][N] double2, lanes N <= kBlock; else the warps' sums
+  // [KG][8 warps][N] float2, N <= 128 with VEC = 4 (8 N <= kBlock with VEC = 1,
+  // where wider rows span warps: [KG][lanes][N])
+  __shared__ double2 buf[KG * kBlock * (VEC == 4 ? 2 : 1)];
+  __shared__ double2 res[KG * (VEC == 4 ? 128 : kBlock)];  // [KG][N]
+  const int k0 = blockIdx.y * KG, ch = blockIdx.x / ranks, rank = blockIdx.x % ranks;
+  const int nk = min(KG, K - k0);
+  size_t r0 = rows * ch / nchunk, r1 = rows * (ch + 1) / nchunk;
+  if (ranks > 1) {
+    const size_t n = r1 - r0, base = r0;
+    r0 = base + n * rank / ranks, r1 = base + n * (rank + 1) / ranks;
+  }
+  const int tid = threadIdx.x, Q = N / VEC, lanes = dot_lanes(Q);
+  const bool warp_rows = Q <= 32;
+  const int lw = warp_rows ? 32 / Q : 1;                      // rows of a warp
+  const int wlane = warp_rows ? (tid & 31) / Q : 0;           // this thread's row among them
+  const int q = warp_rows ? (tid & 31) % Q : tid % Q;
+  const int lane = warp_rows ? (tid >> 5) * lw + wlane : tid / Q;
+  const bool on = warp_rows ? wlane < lw : lane < lanes;
+  double are[FLUSH ? KG : 1][VEC], aim[FLUSH ? KG : 1][VEC];
+  R pre[KG][VEC], pim[KG][VEC];
 #pragma unroll
-  for (int j = 0; j < kKG; ++j)
+  for (int j = 0; j < KG; ++j)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) pre[j][e] = pim[j][e] = 0.f;
-  if (lane < lanes) {
+    for (int e = 0; e < VEC; ++e) {
+      if (FLUSH) are[j][e] = aim[j][e] = 0;
+      pre[j][e] = pim[j][e] = 0;
+    }
+  if (on) {
+    int cnt = 0;
     for (size_t row = r0 + lane; row < r1; row += lanes) {
-      const float4 yr = *reinterpret_cast<const float4*>(Y + fidx(row, 0, N, 4 * q));
-      const float4 yi = *reinterpret_cast<const float4*>(Y + fidx(row, 1, N, 4 * q));
+      R yr[VEC], yi[VEC];
+      ld_row<S, VEC>(Y + fidx(row, 0, N, VEC * q), yr);
+      ld_row<S, VEC>(Y + fidx(row, 1, N, VEC * q), yi);
 #pragma unroll
-      for (int j = 0; j < kKG; ++j) {
+      for (int j = 0; j < KG; ++j) {
         if (j < nk) {
-          const float* Xk = X + (size_t)(k0 + j) * stride;
-          const float4 xr = *reinterpret_cast<const float4*>(Xk + fidx(row, 0, N, 4 * q));
-          const float4 xi = *reinterpret_cast<const float4*>(Xk + fidx(row, 1, N, 4 * q));
-          const float xre[4] = {xr.x, xr.y, xr.z, xr.w}, xim[4] = {xi.x, xi.y, xi.z, xi.w};
-          const float yre[4] = {yr.x, yr.y, yr.z, yr.w}, yim[4] = {yi.x, yi.y, yi.z, yi.w};
+          const S* Xk = X + (size_t)(k0 + j) * stride;
+          R xr[VEC], xi[VEC];
+          ld_row<S, VEC>(Xk + fidx(row, 0, N, VEC * q), xr);
+          ld_row<S, VEC>(Xk + fidx(row, 1, N, VEC * q), xi);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            pre[j][e] = fmaf(xre[e], yre[e], fmaf(xim[e], yim[e], pre[j][e]));
-            pim[j][e] = fmaf(xre[e], yim[e], fmaf(-xim[e], yre[e], pim[j][e]));
+          for (int e = 0; e < VEC; ++e) {
+            pre[j][e] = fma(xr[e], yr[e], fma(xi[e], yi[e], pre[j][e]));
+            pim[j][e] = fma(xr[e], yi[e], fma(-xi[e], yr[e], pim[j][e]));
           }
         }
       }
+      if (FLUSH && ++cnt == kFlush) {
+#pragma unroll
+        for (int j = 0; j < KG; ++j)
+#pragma unroll
+          for (int e = 0; e < VEC; ++e)
+            are[j][e] += pre[j][e], aim[j][e] += pim[j][e], pre[j][e] = pim[j][e] = 0;
+        cnt = 0;
+      }
     }
   }
+  if constexpr (FLUSH) {
+    static_assert(VEC == 1, "lanes * N <= kBlock");
 #pragma unroll
-  for (int j = 0; j < kKG; ++j) {
-    if (j >= nk) break;
-    if (lane < lanes) {
+    for (int j = 0; j < KG; ++j)
+      if (on && j < nk)
+        buf[j * kBlock + lane * N + q] = make_double2(are[j][0] + (double)pre[j][0], aim[j][0] + (double)pim[j][0]);
+    __syncthreads();
+    int half = 1;  // the largest power of two below the number of lanes
+    while (2 * half < lanes) half *= 2;
+    if (lanes > 1)
+      for (int h = half; h > 0; h >>= 1) {
+        for (int e = tid; e < h * N && e + h * N < lanes * N; e += kBlock)
+          for (int j = 0; j < nk; ++j) {
+            double2& t = buf[j * kBlock + e];
+            const double2 o = buf[j * kBlock + e + h * N];
+            t.x += o.x, t.y += o.y;
+          }
+        __syncthreads();
+      }
+    for (int e = tid; e < nk * N; e += kBlock) res[e] = buf[(e / N) * kBlock + e % N];
+  } else {
+    float2* wsum = reinterpret_cast<float2*>(buf);
+    const int units = warp_rows ? kBlock / 32 : lanes, unit = warp_rows ? tid >> 5 : lane;
+    int half = 1;
+    while (2 * half < lw) half *= 2;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        sre[lane * N + 4 * q + e] = (double)pre[j][e];
-        sim[lane * N + 4 * q + e] = (double)pim[j][e];
+    for (int j = 0; j < KG; ++j) {
+      if (j >= nk) break;
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) {
+        float a = pre[j][e], b = pim[j][e];
+        if (lw > 1)
+          for (int h = half; h > 0; h >>= 1) {
+            const float oa = __shfl_down_sync(0xffffffffu, a, h * Q), ob = __shfl_down_sync(0xffffffffu, b, h * Q);
+            if (wlane < h && wlane + h < lw) a += oa, b += ob;
+          }
+        if (on && wlane == 0) wsum[(j * units + unit) * N + VEC * q + e] = make_float2(a, b);
       }
     }
     __syncthreads();
-    if (tid < N) {
-      double a = 0, b = 0;
-      for (int l = 0; l < lanes; ++l) {
-        a += sre[l * N + tid];
-        b += sim[l * N + tid];
-      }
-      double* o = part + (((size_t)(k0 + j) * nchunk + ch) * N + tid) * 2;
-      o[0] = a;
-      o[1] = b;
+    for (int e = tid; e < nk * N; e += kBlock) {
+      const float2* w = wsum + (size_t)(e / N) * units * N + e % N;
+      double2 t = make_double2(0, 0);
+      for (int u = 0; u < units; ++u) t.x += (double)w[u * N].x, t.y += (double)w[u * N].y;
+      res[e] = t;
     }
-    __syncthreads();
   }
+  if (ranks > 1) cg::this_cluster().sync();
+  else __syncthreads();
+  if (rank == 0) {
+    for (int e = tid; e < nk * N; e += kBlock) {
+      double2 t = res[e];
+      for (int c = 1; c < ranks; ++c) {
+        const double2 o = *cg::this_cluster().map_shared_rank(&res[e], c);
+        t.x += o.x, t.y += o.y;
+      }
+      *reinterpret_cast<double2*>(part + (((size_t)(k0 + e / N) * nchunk + ch) * N + e % N) * 2) = t;
+    }
+  }
+  if (ranks > 1) cg::this_cluster().sync();  // the ranks' shared memory stays until it has been read
 }
 
 // out[k][r] = sum over the chunks of part[k][chunk][r]: one warp per (k, r),
 // lane l adds chunks l, l+32, ... and the lanes are joined by a fixed
-// butterfly, so the order of the sum does not depend on timing
-__global__ void k_sum_chunks(const double* part, int K, int nchunk, int N, double* out) {
+// butterfly, so the order of the sum does not depend on timing; out32 (may be
+// null): the same rounded to FP32, the coefficients of a following multi_axpy
+__global__ void k_sum_chunks(const double* part, int K, int nchunk, int N, double* out, float* out32) {
   const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (t >= K * N) return;
   const int k = t / N, r = t % N;
@@ -170,13 +210,14 @@ __global__ void k_sum_chunks(const double* part, int K, int nchunk, int N, doubl
   if (lane == 0) {
     out[2 * t] = a;
     out[2 * t + 1] = b;
+    if (out32) *reinterpret_cast<float2*>(out32 + 2 * t) = make_float2((float)a, (float)b);
   }
 }
 
-// coefficients sign*coef in the compute precision, once per (k, r)
-__global__ void k_coef_to_float(const double* coef, double sign, float* out, int n) {
+// coefficients in the compute precision, once per (k, r)
+__global__ void k_coef_to_float(const double* coef, float* out, int n) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n) out[t] = (float)(sign * coef[t]);
+  if (t < n) out[t] = (float)coef[t];
 }
 
 template <class S, class C>
@@ -201,7 +242,7 @@ __global__ void k_multi_axpy(const S* X, size_t stride, int K, S* Y, size_t rows
 // FP32, N % 4 == 0: four right-hand sides per thread, 16-byte loads and
 // stores (the scalar kernel's operations in its order: the same bits)
 __global__ void k_multi_axpy4(const float* __restrict__ X, size_t stride, int K, float* __restrict__ Y, size_t rows,
-                              int N, const float* __restrict__ coef) {
+                              int N, const float* __restrict__ coef, float sign) {
   const int Q = N / 4;
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (t >= rows * Q) return;
@@ -214,7 +255,8 @@ __global__ void k_multi_axpy4(const float* __restrict__ X, size_t stride, int K,
   for (int k = 0; k < K; ++k) {
     const float4 c01 = *reinterpret_cast<const float4*>(coef + ((size_t)k * N + 4 * q) * 2);
     const float4 c23 = *reinterpret_cast<const float4*>(coef + ((size_t)k * N + 4 * q) * 2 + 4);
-    const float cr[4] = {c01.x, c01.z, c23.x, c23.z}, ci[4] = {c01.y, c01.w, c23.y, c23.w};
+    const float cr[4] = {sign * c01.x, sign * c01.z, sign * c23.x, sign * c23.z};
+    const float ci[4] = {sign * c01.y, sign * c01.w, sign * c23.y, sign * c23.w};
     const float* Xk = X + (size_t)k * stride;
     const float4 x0 = *reinterpret_cast<const float4*>(Xk + fidx(row, 0, N, 4 * q));
     const float4 x1 = *reinterpret_cast<const float4*>(Xk + fidx(row, 1, N, 4 * q));
@@ -252,52 +294,64 @@ __global__ void k_scale_by(S* X, size_t rows, int N, const double* s) {
 
 // the four-RHS kernels need FP32, N % 4 == 0 and 16-byte aligned rows
 bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
-bool use_dot4(const void* X, size_t stride, const void* Y, size_t rows, int N, int dtype, int nch) {
-  if (dtype != MRHS_F32 || N % 4 != 0 || N > 4 * kBlock || !aligned16(X) || !aligned16(Y) || stride % 4 != 0)
-    return false;
-  const size_t lanes = kBlock / (N / 4);
-  return (rows / nch + lanes - 1) / lanes <= (size_t)kMaxRows4;
+bool use_dot4(const void* X, size_t stride, const void* Y, int N, int dtype) {
+  return dtype == MRHS_F32 && N % 4 == 0 && N <= 128 && aligned16(X) && aligned16(Y) && stride % 4 == 0;
 }
 
 }  // namespace
 
-void multi_dot(mrhs_ctx c, const void* X, size_t stride, int K, const void* Y, size_t rows, int N, int dtype,
-               double* out) {
-  MRHS_REQUIRE(N >= 1 && N <= kBlock && K >= 1, MRHS_ERR_ARG, "multi_dot: bad sizes");
-  int nch = n_chunks(rows, N);
-  double* part = (double*)scratch(c, SC_RED, sizeof(double) * 2 * (size_t)K * nch * N);
-  dim3 grid(nch, (K + kKG - 1) / kKG);
-  Prof pr(c, "multi_dot");
-  if (use_dot4(X, stride, Y, rows, N, dtype, nch))
-    k_multi_dot4<<<dim3(nch, (K + kKG4 - 1) / kKG4), kBlock, 0, c->stream>>>((const float*)X, stride, K,
-                                                                             (const float*)Y, rows, N, nch, part);
-  else
-    MRHS_DISPATCH(dtype, S, (k_multi_dot<S><<<grid, kBlock, 0, c->stream>>>((const S*)X, stride, K, (const S*)Y, rows, N, nch, part)));
-  MRHS_LAUNCH_CHECK("multi_dot");
-  k_sum_chunks<<<grid_for((size_t)K * N * 32, 256), 256, 0, c->stream>>>(part, K, nch, N, out);
-  MRHS_LAUNCH_CHECK("sum_chunks");
+namespace {
+template <class S>
+auto dot_kernel(bool flush) {
+  if constexpr (sizeof(S) < 8)
+    if (!flush) return k_multi_dot<S, 1, kKG, false>;
+  return k_multi_dot<S, 1, kKG, true>;
 }
+}  // namespace
 
-// multi_dot with the per-CTA partials in a caller-supplied buffer of at
-// least multi_dot_partials_bytes(rows, N, K) bytes (no allocation)
 size_t multi_dot_partials_bytes(size_t rows, int N, int K) {
   return sizeof(double) * 2 * (size_t)K * n_chunks(rows, N) * N;
 }
 
+// part: a buffer of multi_dot_partials_bytes(rows, N, K) bytes
 void multi_dot_ws(mrhs_ctx c, const void* X, size_t stride, int K, const void* Y, size_t rows, int N, int dtype,
-                  double* out, double* part) {
+                  double* out, double* part, float* out32) {
   MRHS_REQUIRE(N >= 1 && N <= kBlock && K >= 1, MRHS_ERR_ARG, "multi_dot: bad sizes");
-  int nch = n_chunks(rows, N);
-  dim3 grid(nch, (K + kKG - 1) / kKG);
+  const int nch = n_chunks(rows, N);
+  const bool four = use_dot4(X, stride, Y, N, dtype);
+  // rows that a thread would sum with one CTA per chunk
+  auto thread_rows = [&](int vec) { return (rows / nch) / dot_lanes(N / vec) + 1; };
+  const bool four_ok = four && thread_rows(4) <= kMaxRows;
+  const int groups = (K + kKG - 1) / kKG;
+  const int ranks = nch * groups < kClusterBelow ? kClusterCtas : 1;
+  const bool flush = dtype == MRHS_F64 || thread_rows(1) > kMaxRows;
   Prof pr(c, "multi_dot");
-  if (use_dot4(X, stride, Y, rows, N, dtype, nch))
-    k_multi_dot4<<<dim3(nch, (K + kKG4 - 1) / kKG4), kBlock, 0, c->stream>>>((const float*)X, stride, K,
-                                                                             (const float*)Y, rows, N, nch, part);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nch * ranks, groups);
+  cfg.blockDim = dim3(kBlock);
+  cfg.stream = c->stream;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = ranks, at.val.clusterDim.y = 1, at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = ranks > 1 ? 1 : 0;
+  if (four_ok)
+    MRHS_CUDA(cudaLaunchKernelEx(&cfg, k_multi_dot<float, 4, kKG, false>, (const float*)X, stride, K, (const float*)Y,
+                                 rows, N, nch, ranks, part));
   else
-    MRHS_DISPATCH(dtype, S, (k_multi_dot<S><<<grid, kBlock, 0, c->stream>>>((const S*)X, stride, K, (const S*)Y, rows, N, nch, part)));
+    MRHS_DISPATCH(dtype, S, {
+      MRHS_CUDA(cudaLaunchKernelEx(&cfg, dot_kernel<S>(flush), (const S*)X, stride, K, (const S*)Y, rows, N, nch, ranks, part));
+    });
   MRHS_LAUNCH_CHECK("multi_dot");
-  k_sum_chunks<<<grid_for((size_t)K * N * 32, 256), 256, 0, c->stream>>>(part, K, nch, N, out);
+  k_sum_chunks<<<grid_for((size_t)K * N * 32, 256), 256, 0, c->stream>>>(part, K, nch, N, out, out32);
   MRHS_LAUNCH_CHECK("sum_chunks");
+}
+
+void multi_dot(mrhs_ctx c, const void* X, size_t stride, int K, const void* Y, size_t rows, int N, int dtype,
+               double* out, float* out32) {
+  MRHS_REQUIRE(N >= 1 && N <= kBlock && K >= 1, MRHS_ERR_ARG, "multi_dot: bad sizes");
+  double* part = (double*)scratch(c, SC_RED, multi_dot_partials_bytes(rows, N, K));
+  multi_dot_ws(c, X, stride, K, Y, rows, N, dtype, out, part, out32);
 }
 
 // out[r] (as [N][2], imaginary part 0) = |X_r|^2
@@ -305,21 +359,27 @@ void norms(mrhs_ctx c, const void* X, size_t rows, int N, int dtype, double* out
   multi_dot(c, X, 0, 1, X, rows, N, dtype, out);
 }
 
+// coef32 (may be null): the coefficients in FP32 as a multi_dot has left them;
+// otherwise they are converted here
 void multi_axpy(mrhs_ctx c, const void* X, size_t stride, int K, void* Y, size_t rows, int N, int dtype,
-                const double* coef, double sign) {
+                const double* coef, double sign, const float* coef32) {
   size_t work = rows * N;
   Prof pr(c, "multi_axpy");
   if (dtype == MRHS_F64) {
     k_multi_axpy<double, double><<<grid_for(work, kBlock), kBlock, 0, c->stream>>>((const double*)X, stride, K, (double*)Y, rows, N, coef, sign);
   } else {
     MRHS_REQUIRE(K <= 65 && N <= 256, MRHS_ERR_ARG, "multi_axpy: K <= 65 and N <= 256");
-    const int n = 2 * K * N;
-    k_coef_to_float<<<grid_for(n, 256), 256, 0, c->stream>>>(coef, sign, c->coef32, n);
+    if (!coef32) {
+      const int n = 2 * K * N;
+      k_coef_to_float<<<grid_for(n, 256), 256, 0, c->stream>>>(coef, c->coef32, n);
+      coef32 = c->coef32;
+    }
+    const float sg = sign < 0 ? -1.f : 1.f;
     if (dtype == MRHS_F32 && N % 4 == 0 && aligned16(X) && aligned16(Y) && stride % 4 == 0)
       k_multi_axpy4<<<grid_for(rows * (N / 4), kBlock), kBlock, 0, c->stream>>>((const float*)X, stride, K, (float*)Y,
-                                                                                rows, N, (const float*)c->coef32);
+                                                                                rows, N, coef32, sg);
     else
-      MRHS_DISPATCH(dtype, S, (k_multi_axpy<S, float><<<grid_for(work, kBlock), kBlock, 0, c->stream>>>((const S*)X, stride, K, (S*)Y, rows, N, (const float*)c->coef32, 1.0f)));
+      MRHS_DISPATCH(dtype, S, (k_multi_axpy<S, float><<<grid_for(work, kBlock), kBlock, 0, c->stream>>>((const S*)X, stride, K, (S*)Y, rows, N, coef32, sg)));
   }
   MRHS_LAUNCH_CHECK("multi_axpy");
 }

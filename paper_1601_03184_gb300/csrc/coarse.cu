@@ -1256,10 +1256,10 @@ static void coarse_gmres(mrhs_ctx c, const void* bc, void* xc, int N, int dtype,
     int kmax = 0;
     for (int k = 0; k < m; ++k) {
       op(Vk(k), w);
-      multi_dot(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1);
-      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, -1.0);
-      multi_dot(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2);
-      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, -1.0);
+      multi_dot(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, c->coef32);
+      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, -1.0, c->coef32);
+      multi_dot(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, c->coef32);
+      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, -1.0, c->coef32);
       norms(c, w, rows, N, dtype, st.hn2);
       MRHS_CUDA(cudaMemsetAsync(st.counter, 0, sizeof(int), c->stream));
       k_gm_step<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N, m, k, tol, maxit);
@@ -1409,10 +1409,10 @@ void coarse_solve_ws(mrhs_ctx c, const void* bc, void* xc, int N, int dtype, dou
     int kmax = 0;
     for (int k = 0; k < m; ++k) {
       apply_Dc(c, Vk(k), w, N, dtype);
-      multi_dot_ws(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, part);
-      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, -1.0);
-      multi_dot_ws(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, part);
-      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, -1.0);
+      multi_dot_ws(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, part, c->coef32);
+      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, -1.0, c->coef32);
+      multi_dot_ws(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, part, c->coef32);
+      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, -1.0, c->coef32);
       multi_dot_ws(c, w, 0, 1, w, rows, N, dtype, st.hn2, part);
       MRHS_CUDA(cudaMemsetAsync(st.counter, 0, sizeof(int), c->stream));
       k_gm_step<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N, m, k, tol, maxit);

@@ -321,7 +321,7 @@ void coarse_solve(mrhs_ctx c, const void* bc, void* xc, int nrhs, int dtype, dou
 // blas.cu: per right-hand-side reductions and updates on interleaved arrays of
 // `rows` complex rows, each [2][N]
 void multi_dot(mrhs_ctx c, const void* X, size_t stride, int K, const void* Y, size_t rows, int N, int dtype,
-               double* out /* device [K][N][2] */);
+               double* out /* device [K][N][2] */, float* out32 = nullptr /* the same in FP32 */);
 void norms(mrhs_ctx c, const void* X, size_t rows, int N, int dtype, double* out /* device [N] (squared) */);
 void convert(mrhs_ctx c, const void* x, int dx, void* y, int dy, size_t n);
 void convert_scaled(mrhs_ctx c, const void* x, int dx, void* y, int dy, size_t n, float scale);
@@ -345,11 +345,11 @@ void sap_pk(mrhs_ctx c, const void* b, int bdtype, void* x, int nrhs, int n_swee
 void sap_tm(mrhs_ctx c, const void* b, int bdtype, void* x, int nrhs, int n_sweeps, int n_mr);
 // blas.cu: y[row][r] += sign * sum_k coef[k][r] * X_k[row][r], X_k = X + k*stride elements
 void multi_axpy(mrhs_ctx c, const void* X, size_t stride, int K, void* Y, size_t rows, int N, int dtype,
-                const double* coef /* device [K][N][2] */, double sign);
+                const double* coef /* device [K][N][2] */, double sign /* 1 or -1 */, const float* coef32 = nullptr);
 void normalise_rhs(mrhs_ctx c, void* X, size_t rows, int N, int dtype);
 size_t multi_dot_partials_bytes(size_t rows, int N, int K);
 void multi_dot_ws(mrhs_ctx c, const void* X, size_t stride, int K, const void* Y, size_t rows, int N, int dtype,
-                  double* out, double* part);
+                  double* out, double* part, float* out32 = nullptr);
 // coarse.cu: the coarse solve on a caller-supplied workspace (no allocation)
 size_t coarse_solve_ws_bytes(mrhs_ctx c, int nrhs, int dtype, int restart);
 void coarse_solve_ws(mrhs_ctx c, const void* bc, void* xc, int nrhs, int dtype, double tol, int restart, int maxit,

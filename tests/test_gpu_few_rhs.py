@@ -41,3 +41,31 @@ def test_coarse_stencil_of_few_vectors(ntv, prec):
         err = np.abs(lat.to_host(yd, nrhs, wd, coarse=True) - ref)
         assert np.all(err <= 2 ** 0.5 * n * u / (1 - n * u) * size + 1e-300), nrhs
     lat.close()
+
+
+# The reductions of the coarse GMRES at the edges of their forms: four right-hand
+# sides per thread (4, 12, 20: rows joined in a warp; 128: a row is a whole warp),
+# one per thread (1, 3, 33, 132: a row spans warps), each as a cluster of CTAs
+# per chunk (1024 and 32768 rows of 256 aggregates are few); seven steps with a
+# restart after five. The oracle's solve of the same D_c; bounds of the coarse
+# solve's other parity tests.
+@pytest.mark.parametrize("prec,tol", [(MRHS_PREC_FP32, 2e-5), (MRHS_PREC_FP64, 1e-10)])
+@pytest.mark.parametrize("nrhs", [1, 3, 4, 12, 20, 33, 128, 132])
+def test_coarse_gmres_reductions(nrhs, prec, tol):
+    dims, agg, ntv = (8, 8, 8, 8), (2, 2, 2, 2), 2
+    wd = MRHS_F32 if prec == MRHS_PREC_FP32 else MRHS_F64
+    lat = Lattice(dims, agg, ntv, prec)
+    lat.set_gauge(inputs.gauge_field(dims, 0.5, 1402))
+    lat.build_clover(0.1, 1.2)
+    lat.set_tv(lat.to_device(inputs.test_vectors(ntv, dims, 2402), wd), wd)
+    lat.build_P()
+    lat.build_Dc()
+    b = inputs.gaussian_field((nrhs, lat.nagg, 2 * ntv), 4402)
+    xd = lat.field(nrhs, wd, coarse=True)
+    its = lat.coarse_solve(lat.to_device(b, wd, coarse=True), xd, nrhs, wd, 0.0, 5, 7)
+    ref, rits = oracle.coarse_solve(dims, agg, lat.get_Dc(), b, 0.0, 5, 7)
+    x = lat.to_host(xd, nrhs, wd, coarse=True)
+    assert list(its) == list(rits)
+    for r in range(nrhs):
+        assert np.linalg.norm(x[r] - ref[r]) <= tol * np.linalg.norm(ref[r]), r
+    lat.close()
