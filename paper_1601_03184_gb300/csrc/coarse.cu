@@ -1,6 +1,7 @@
 // Coarse grid: D_c = P^dag D P assembly, restriction R = P^dag (Algorithm 3
 // of the paper, all right-hand sides at once), prolongation, the coarse
 // 9-point stencil and the multi-RHS coarse GMRES.
+#include <algorithm>
 #include <cstdint>
 #include <cstdlib>
 
@@ -602,6 +603,16 @@ __global__ void k_scale_rhs(const S* x, S* y, size_t rows, int N, const double* 
   y[fidx(row, 1, N, r)] = from_r<S>(to_r(x[fidx(row, 1, N, r)]) * f);
 }
 
+// the same four right-hand sides at a time (FP32, N % 4 == 0, 16-byte rows)
+__global__ void k_scale_rhs4(const float4* __restrict__ x, float4* __restrict__ y, size_t n4, int N,
+                             const double* __restrict__ s) {
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (t >= n4) return;
+  const int r = 4 * (int)(t % (size_t)(N / 4));
+  const float4 v = x[t];
+  y[t] = make_float4(v.x * (float)s[r], v.y * (float)s[r + 1], v.z * (float)s[r + 2], v.w * (float)s[r + 3]);
+}
+
 // ------------------------------------------------------- GMRES state ------
 struct GmState {
   cx<double>* H;    // [N][m+1][m]
@@ -619,7 +630,7 @@ struct GmState {
   int* active;      // [N]
   int* its;         // [N]
   int* kend;        // [N]
-  int* counter;     // [1]
+  int* counter;     // [2]: active right-hand sides and finished CTAs of a step (both zero between launches)
 };
 
 __global__ void k_gm_init(GmState st, int N) {
@@ -631,92 +642,121 @@ __global__ void k_gm_init(GmState st, int N) {
   st.kend[r] = 0;
 }
 
-// start of a cycle: r = b - A x is in w with |w|^2 in beta2
-__global__ void k_gm_start(GmState st, int N, int m, double tol, int maxit) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= N) return;
-  st.kend[r] = 0;
-  st.active[r] = 0;
-  st.inv[r] = 0;
-  if (st.conv[r] || st.its[r] >= maxit) return;
-  double beta = sqrt(st.beta2[2 * r]);
-  if (beta <= tol * sqrt(st.bnorm2[2 * r])) {
-    st.conv[r] = 1;
-    return;
+// start of a cycle: r = b - A x has the squared norms beta2; *hcount (pinned
+// host memory) receives the number of right-hand sides that go on (one CTA)
+__global__ void __launch_bounds__(256) k_gm_start(GmState st, const double* beta2, int N, int m, double tol, int maxit,
+                                                  int* hcount) {
+  const int r = threadIdx.x;
+  bool on = false;
+  if (r < N) {
+    st.kend[r] = 0;
+    st.active[r] = 0;
+    st.inv[r] = 0;
+    if (!st.conv[r] && st.its[r] < maxit) {
+      const double beta = sqrt(beta2[2 * r]);
+      if (beta <= tol * sqrt(st.bnorm2[2 * r])) {
+        st.conv[r] = 1;
+      } else {
+        on = true;
+        st.active[r] = 1;
+        st.inv[r] = 1.0 / beta;
+        for (int i = 0; i <= m; ++i) st.g[(size_t)r * (m + 1) + i] = mk(0.0, 0.0);
+        st.g[(size_t)r * (m + 1)] = mk(beta, 0.0);
+      }
+    }
   }
-  st.active[r] = 1;
-  st.inv[r] = 1.0 / beta;
-  for (int i = 0; i <= m; ++i) st.g[(size_t)r * (m + 1) + i] = mk(0.0, 0.0);
-  st.g[(size_t)r * (m + 1)] = mk(beta, 0.0);
-  atomicAdd(st.counter, 1);
+  const int n = __syncthreads_count(on);
+  if (r == 0) {
+    st.counter[0] = st.counter[1] = 0;
+    *hcount = n;
+    __threadfence_system();
+  }
 }
 
 // Arnoldi column k: h = h1 + h2 (two classical Gram-Schmidt passes), then
-// the Givens rotations and the residual estimate |g_{k+1}|
-__global__ void k_gm_step(GmState st, int N, int m, int k, double tol, int maxit) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= N) return;
-  st.inv[r] = 0;
-  if (!st.active[r]) return;
-  cx<double>* H = st.H + (size_t)r * (m + 1) * m;
-  cx<double>* cs = st.cs + (size_t)r * m;
-  cx<double>* sn = st.sn + (size_t)r * m;
-  cx<double>* g = st.g + (size_t)r * (m + 1);
-  for (int i = 0; i <= k; ++i)
-    H[i * m + k] = mk(st.h1[((size_t)i * N + r) * 2] + st.h2[((size_t)i * N + r) * 2],
-                      st.h1[((size_t)i * N + r) * 2 + 1] + st.h2[((size_t)i * N + r) * 2 + 1]);
-  double hk1 = sqrt(st.hn2[2 * r]);
-  H[(k + 1) * m + k] = mk(hk1, 0.0);
-  for (int i = 0; i < k; ++i) {
-    cx<double> a = H[i * m + k], b = H[(i + 1) * m + k];
-    H[i * m + k] = cnj(cs[i]) * a + cnj(sn[i]) * b;
-    H[(i + 1) * m + k] = mk(0.0, 0.0) - sn[i] * a + cs[i] * b;
+// the Givens rotations and the residual estimate |g_{k+1}|. One warp per
+// right-hand side: its lanes fetch the column and the rotations together (the
+// loads, not the FP64 chain of the rotations, took the time with one thread:
+// 21 us a step on average at k up to 20), lane 0 applies them. The last CTA to finish
+// hands the number of right-hand sides that go on to the host (*hcount, pinned).
+__global__ void __launch_bounds__(32) k_gm_step(GmState st, int N, int m, int k, double tol, int maxit, int* hcount) {
+  __shared__ cx<double> sh[65], sc[64], ss[64];
+  const int r = blockIdx.x, lane = threadIdx.x;
+  int on = 0;
+  if (st.active[r]) {
+    cx<double>* H = st.H + (size_t)r * (m + 1) * m;
+    cx<double>* cs = st.cs + (size_t)r * m;
+    cx<double>* sn = st.sn + (size_t)r * m;
+    cx<double>* g = st.g + (size_t)r * (m + 1);
+    for (int i = lane; i <= k; i += 32) {
+      const double2 a = *reinterpret_cast<const double2*>(st.h1 + ((size_t)i * N + r) * 2);
+      const double2 b = *reinterpret_cast<const double2*>(st.h2 + ((size_t)i * N + r) * 2);
+      sh[i] = mk(a.x + b.x, a.y + b.y);
+      if (i < k) sc[i] = cs[i], ss[i] = sn[i];
+    }
+    const cx<double> g0 = g[k];
+    const double hk1 = sqrt(st.hn2[2 * r]), goal = tol * sqrt(st.bnorm2[2 * r]);
+    const int its = st.its[r] + 1;
+    __syncwarp();
+    if (lane == 0) {
+      cx<double> a = sh[0];
+      for (int i = 0; i < k; ++i) {
+        const cx<double> b = sh[i + 1];
+        sh[i] = cnj(sc[i]) * a + cnj(ss[i]) * b;
+        a = mk(0.0, 0.0) - ss[i] * a + sc[i] * b;
+      }
+      const double nu = sqrt(a.re * a.re + a.im * a.im + hk1 * hk1);
+      const cx<double> ck = nu == 0 ? mk(1.0, 0.0) : scale(a, 1.0 / nu);
+      const cx<double> sk = nu == 0 ? mk(0.0, 0.0) : mk(hk1 * (1.0 / nu), 0.0);
+      sh[k] = mk(nu, 0.0);
+      cs[k] = ck;
+      sn[k] = sk;
+      const cx<double> g1 = mk(0.0, 0.0) - sk * g0;
+      g[k] = cnj(ck) * g0;
+      g[k + 1] = g1;
+      st.its[r] = its;
+      st.kend[r] = k + 1;
+      const double res = sqrt(g1.re * g1.re + g1.im * g1.im);
+      const bool conv = res <= goal || hk1 == 0;
+      if (conv) st.conv[r] = 1;
+      on = !(conv || its >= maxit || k + 1 == m);
+      st.active[r] = on;
+      st.inv[r] = on ? 1.0 / hk1 : 0.0;
+    }
+    __syncwarp();
+    for (int i = lane; i <= k; i += 32) H[i * m + k] = sh[i];
+  } else if (lane == 0) {
+    st.inv[r] = 0;
   }
-  cx<double> a = H[k * m + k], b = H[(k + 1) * m + k];
-  double nu = sqrt(a.re * a.re + a.im * a.im + b.re * b.re + b.im * b.im);
-  if (nu == 0) {
-    cs[k] = mk(1.0, 0.0);
-    sn[k] = mk(0.0, 0.0);
-  } else {
-    cs[k] = scale(a, 1.0 / nu);
-    sn[k] = scale(b, 1.0 / nu);
-  }
-  H[k * m + k] = mk(nu, 0.0);
-  H[(k + 1) * m + k] = mk(0.0, 0.0);
-  cx<double> g0 = g[k];
-  g[k] = cnj(cs[k]) * g0;
-  g[k + 1] = mk(0.0, 0.0) - sn[k] * g0;
-  st.its[r] += 1;
-  st.kend[r] = k + 1;
-  double res = sqrt(g[k + 1].re * g[k + 1].re + g[k + 1].im * g[k + 1].im);
-  bool conv = res <= tol * sqrt(st.bnorm2[2 * r]) || hk1 == 0;
-  if (conv) st.conv[r] = 1;
-  if (conv || st.its[r] >= maxit || k + 1 == m) {
-    st.active[r] = 0;
-  } else {
-    st.inv[r] = 1.0 / hk1;
-    atomicAdd(st.counter, 1);
+  if (lane == 0) {
+    if (on) atomicAdd(st.counter, 1);
+    __threadfence();
+    if (atomicAdd(st.counter + 1, 1) == gridDim.x - 1) {
+      *hcount = atomicExch(st.counter, 0);
+      st.counter[1] = 0;
+      __threadfence_system();
+    }
   }
 }
 
-// back substitution of the leading kend x kend triangle, y = coefficients
-__global__ void k_gm_solve(GmState st, int N, int m) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= N) return;
+// back substitution of the leading kend x kend triangle, y = coefficients;
+// one CTA per right-hand side, thread l keeps row l of the right side
+__global__ void __launch_bounds__(64) k_gm_solve(GmState st, int N, int m) {
+  __shared__ cx<double> sy;
+  const int r = blockIdx.x, l = threadIdx.x;
   const cx<double>* H = st.H + (size_t)r * (m + 1) * m;
-  const cx<double>* g = st.g + (size_t)r * (m + 1);
-  int ke = st.kend[r];
-  cx<double> yv[64];
+  const int ke = st.kend[r];
+  cx<double> c = l < ke ? st.g[(size_t)r * (m + 1) + l] : mk(0.0, 0.0);
   for (int i = ke - 1; i >= 0; --i) {
-    cx<double> c = g[i];
-    for (int l = i + 1; l < ke; ++l) c = c - H[i * m + l] * yv[l];
-    double d = H[i * m + i].re;  // real and positive after the rotation
-    yv[i] = scale(c, 1.0 / d);
+    const cx<double> h = l <= i ? H[l * m + i] : mk(0.0, 0.0);  // real and positive for l = i
+    if (l == i) sy = c = scale(c, 1.0 / h.re);
+    __syncthreads();
+    if (l < i) c = c - h * sy;
+    __syncthreads();
   }
-  for (int i = 0; i < m; ++i) {
-    cx<double> v = i < ke ? yv[i] : mk(0.0, 0.0);
-    st.y[((size_t)i * N + r) * 2] = v.re;
-    st.y[((size_t)i * N + r) * 2 + 1] = v.im;
+  if (l < m) {
+    st.y[((size_t)l * N + r) * 2] = c.re;
+    st.y[((size_t)l * N + r) * 2 + 1] = c.im;
   }
 }
 
@@ -1199,19 +1239,13 @@ static void apply_schur(mrhs_ctx c, const void* x, void* y, void* t, void* u, in
   apply_Dc_part(c, colour_part(c, 0, 0, x, u, nullptr), y, N, dtype);
 }
 
-// restarted GMRES on `rows` coarse rows: op(x, y) is D_c, or S on compact
-// even fields
-template <class Op>
-static void coarse_gmres(mrhs_ctx c, const void* bc, void* xc, int N, int dtype, double tol, int m, int maxit,
-                         int* iters, size_t rows, Op op) {
-  const size_t fe = rows * 2 * N;  // elements of one coarse field
-  const size_t es = dtype_size(dtype);
-  char* basis = (char*)scratch(c, SC_KRYLOV, (size_t)(m + 2) * fe * es);
-  char* w = basis + (size_t)(m + 1) * fe * es;
-  auto Vk = [&](int k) { return (void*)(basis + (size_t)k * fe * es); };
-  size_t sbytes = 0;
-  sbytes += 3 * sizeof(cx<double>) * N * (size_t)(m + 1) * m + 256 * 16;
-  char* sp = (char*)scratch(c, SC_HESS, sbytes + sizeof(double) * 16 * N * (size_t)(m + 2) + 4096);
+// The workspace of one restarted GMRES: basis V_0..V_m and w, state, partials
+struct GmSpace {
+  char* basis;
+  GmState st;
+  double* part;
+};
+static GmState carve_state(char* sp, int N, int m) {
   GmState st;
   st.H = carve<cx<double>>(sp, (size_t)N * (m + 1) * m);
   st.cs = carve<cx<double>>(sp, (size_t)N * m);
@@ -1228,56 +1262,114 @@ static void coarse_gmres(mrhs_ctx c, const void* bc, void* xc, int N, int dtype,
   st.active = carve<int>(sp, N);
   st.its = carve<int>(sp, N);
   st.kend = carve<int>(sp, N);
-  st.counter = carve<int>(sp, 1);
-  int* hcount = c->hflag + 1;
-  auto read_counter = [&]() {
-    MRHS_CUDA(cudaMemcpyAsync(hcount, st.counter, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    MRHS_CUDA(cudaStreamSynchronize(c->stream));
-    return *hcount;
+  st.counter = carve<int>(sp, 2);
+  return st;
+}
+
+// Vectors up to this size let the host run one Arnoldi step ahead of the
+// convergence count: a step of small vectors is a chain of short launches (some
+// 60 us at 4 MB), and waiting for its count leaves the GPU idle for 10 to 20 us
+// each time, while the step that may be launched in vain after the last one
+// (it changes no result) costs one step. Larger vectors wait: a step at
+// 48^3 x 96 takes 6 ms.
+constexpr size_t kRunAheadBytes = (size_t)16 << 20;
+
+// restarted GMRES on `rows` coarse rows: op(x, y) is D_c, or S on compact
+// even fields
+template <class Op>
+static void coarse_gmres(mrhs_ctx c, const void* bc, void* xc, int N, int dtype, double tol, int m, int maxit,
+                         int* iters, size_t rows, const GmSpace& ws, Op op) {
+  const size_t fe = rows * 2 * N;  // elements of one coarse field
+  const size_t es = dtype_size(dtype);
+  const GmState& st = ws.st;
+  char* w = ws.basis + (size_t)(m + 1) * fe * es;
+  auto Vk = [&](int k) { return (void*)(ws.basis + (size_t)k * fe * es); };
+  auto dots = [&](int K, double* out, float* out32) {
+    multi_dot_ws(c, Vk(0), fe, K, w, rows, N, dtype, out, ws.part, out32);
   };
+  auto norm2 = [&](const void* x, double* out) { multi_dot_ws(c, x, 0, 1, x, rows, N, dtype, out, ws.part); };
   auto scale_into = [&](const void* x, void* y) {
-    MRHS_DISPATCH(dtype, S, (k_scale_rhs<S><<<grid_for(rows * N, 256), 256, 0, c->stream>>>((const S*)x, (S*)y, rows, N, st.inv)));
+    if (dtype == MRHS_F32 && N % 4 == 0 && ((uintptr_t)x & 15) == 0 && ((uintptr_t)y & 15) == 0)
+      k_scale_rhs4<<<grid_for(fe / 4, 256), 256, 0, c->stream>>>((const float4*)x, (float4*)y, fe / 4, N, st.inv);
+    else
+      MRHS_DISPATCH(dtype, S, (k_scale_rhs<S><<<grid_for(rows * N, 256), 256, 0, c->stream>>>((const S*)x, (S*)y, rows, N, st.inv)));
     MRHS_LAUNCH_CHECK("scale_rhs");
   };
+  // the counts of the right-hand sides that go on: one pinned word and one
+  // event per step, two of each in turn
+  for (auto& e : c->gm_event)
+    if (!e) MRHS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  int* hcount = c->hflag + 8;
+  const bool ahead = fe * es <= kRunAheadBytes;
+  int marks = 0;  // counts asked for so far
+  auto mark = [&] { MRHS_CUDA(cudaEventRecord(c->gm_event[marks++ & 1], c->stream)); };
+  auto count_of = [&](int i) {
+    MRHS_CUDA(cudaEventSynchronize(c->gm_event[i & 1]));
+    return *(volatile int*)(hcount + (i & 1));
+  };
   MRHS_CUDA(cudaMemsetAsync(xc, 0, fe * es, c->stream));
-  norms(c, bc, rows, N, dtype, st.bnorm2);
+  norm2(bc, st.bnorm2);
   k_gm_init<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N);
   MRHS_LAUNCH_CHECK("gm_init");
-  for (;;) {
-    op(xc, w);
-    MRHS_DISPATCH(dtype, S, (k_sub_from<S><<<grid_for(fe, 256), 256, 0, c->stream>>>((const S*)bc, (S*)w, fe)));
-    MRHS_LAUNCH_CHECK("sub_from");
-    norms(c, w, rows, N, dtype, st.beta2);
-    MRHS_CUDA(cudaMemsetAsync(st.counter, 0, sizeof(int), c->stream));
-    k_gm_start<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N, m, tol, maxit);
-    MRHS_LAUNCH_CHECK("gm_start");
-    if (read_counter() == 0) break;
-    scale_into(w, Vk(0));
-    int kmax = 0;
-    for (int k = 0; k < m; ++k) {
-      op(Vk(k), w);
-      multi_dot(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, c->coef32);
-      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, -1.0, c->coef32);
-      multi_dot(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, c->coef32);
-      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, -1.0, c->coef32);
-      norms(c, w, rows, N, dtype, st.hn2);
-      MRHS_CUDA(cudaMemsetAsync(st.counter, 0, sizeof(int), c->stream));
-      k_gm_step<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N, m, k, tol, maxit);
-      MRHS_LAUNCH_CHECK("gm_step");
-      kmax = k + 1;
-      int more = read_counter();
-      if (more == 0) break;
-      scale_into(w, Vk(k + 1));
+  // a right-hand side that is still active has taken every step so far, so
+  // none is after maxit steps
+  for (int done = 0; done < maxit;) {
+    const bool first = done == 0;  // x = 0: the residual is b
+    if (!first) {
+      op(xc, w);
+      MRHS_DISPATCH(dtype, S, (k_sub_from<S><<<grid_for(fe, 256), 256, 0, c->stream>>>((const S*)bc, (S*)w, fe)));
+      MRHS_LAUNCH_CHECK("sub_from");
+      norm2(w, st.beta2);
     }
-    k_gm_solve<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N, m);
+    k_gm_start<<<1, 256, 0, c->stream>>>(st, first ? st.bnorm2 : st.beta2, N, m, tol, maxit, hcount + (marks & 1));
+    MRHS_LAUNCH_CHECK("gm_start");
+    mark();
+    if (!ahead && count_of(marks - 1) == 0) break;
+    scale_into(first ? bc : w, Vk(0));
+    const int steps = std::min(m, maxit - done);
+    int kmax = 0;      // columns that count
+    bool more = true;  // right-hand sides left after kmax columns
+    for (int k = 0; k < steps && more; ++k) {
+      op(Vk(k), w);
+      dots(k + 1, st.h1, c->coef32);
+      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, -1.0, c->coef32);
+      dots(k + 1, st.h2, c->coef32);
+      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, -1.0, c->coef32);
+      norm2(w, st.hn2);
+      k_gm_step<<<N, 32, 0, c->stream>>>(st, N, m, k, tol, maxit, hcount + (marks & 1));
+      MRHS_LAUNCH_CHECK("gm_step");
+      mark();
+      // running ahead: the count before this step says whether it counts
+      if (ahead && count_of(marks - 2) == 0) {
+        more = false;
+        break;
+      }
+      kmax = k + 1;
+      if (!ahead) more = count_of(marks - 1) != 0;
+      if (more && k + 1 < steps) scale_into(w, Vk(k + 1));
+    }
+    if (kmax == 0) break;  // nothing went on at the start of the cycle
+    done += kmax;
+    k_gm_solve<<<N, 64, 0, c->stream>>>(st, N, m);
     MRHS_LAUNCH_CHECK("gm_solve");
     multi_axpy(c, Vk(0), fe, kmax, xc, rows, N, dtype, st.y, 1.0);
+    if (kmax < steps) break;  // all have converged
   }
   if (iters) {
     MRHS_CUDA(cudaMemcpyAsync(iters, st.its, sizeof(int) * N, cudaMemcpyDeviceToHost, c->stream));
     MRHS_CUDA(cudaStreamSynchronize(c->stream));
   }
   check_tc_timeout(c);
+}
+
+// the workspace in the context's scratch buffers
+static GmSpace scratch_space(mrhs_ctx c, size_t rows, int N, int dtype, int m) {
+  GmSpace ws;
+  ws.basis = (char*)scratch(c, SC_KRYLOV, (size_t)(m + 2) * rows * 2 * N * dtype_size(dtype));
+  const size_t sbytes = 3 * sizeof(cx<double>) * N * (size_t)(m + 1) * m + 256 * 16;
+  ws.st = carve_state((char*)scratch(c, SC_HESS, sbytes + sizeof(double) * 16 * N * (size_t)(m + 2) + 4096), N, m);
+  ws.part = (double*)scratch(c, SC_RED, multi_dot_partials_bytes(rows, N, m + 1));
+  return ws;
 }
 
 void coarse_solve(mrhs_ctx c, const void* bc, void* xc, int N, int dtype, double tol, int m, int maxit, int* iters) {
@@ -1287,7 +1379,8 @@ void coarse_solve(mrhs_ctx c, const void* bc, void* xc, int N, int dtype, double
                "coarse solve: need 1 <= nrhs <= 256, 1 <= restart <= 64, maxit >= 0, tol >= 0");
   const int nc = 2 * c->ntv;
   if (!c->coarse_eo) {
-    coarse_gmres(c, bc, xc, N, dtype, tol, m, maxit, iters, (size_t)c->g.nagg * nc,
+    const size_t rows = (size_t)c->g.nagg * nc;
+    coarse_gmres(c, bc, xc, N, dtype, tol, m, maxit, iters, rows, scratch_space(c, rows, N, dtype, m),
                  [&](const void* x, void* y) { apply_Dc(c, x, y, N, dtype); });
     return;
   }
@@ -1307,7 +1400,8 @@ void coarse_solve(mrhs_ctx c, const void* bc, void* xc, int N, int dtype, double
   inverse_apply(c, bo, nullptr, u, -1.0, N, dtype);
   apply_Dc_part(c, colour_part(c, 0, 1, nullptr, u, be), bh, N, dtype);
   // GMRES on S from x_e = 0
-  coarse_gmres(c, bh, xe, N, dtype, tol, m, maxit, iters, (size_t)c->ncol[0] * nc,
+  const size_t rows = (size_t)c->ncol[0] * nc;
+  coarse_gmres(c, bh, xe, N, dtype, tol, m, maxit, iters, rows, scratch_space(c, rows, N, dtype, m),
                [&](const void* x, void* y) { apply_schur(c, x, y, t, u, N, dtype); });
   // x_o = D_oo^-1 (b_o - D_oe x_e)
   apply_Dc_part(c, colour_part(c, 1, 1, nullptr, xe, nullptr), t, N, dtype);
@@ -1357,79 +1451,12 @@ void coarse_solve_ws(mrhs_ctx c, const void* bc, void* xc, int N, int dtype, dou
                "coarse solve: need 1 <= nrhs <= 256, 1 <= restart <= 64, maxit >= 0, tol >= 0");
   const WsLayout L = ws_layout(c, N, dtype, m);
   MRHS_REQUIRE(L.total <= ws_bytes, MRHS_ERR_SHAPE, "coarse solve workspace too small");
-  const size_t rows = (size_t)c->g.nagg * 2 * c->ntv;
-  const size_t fe = rows * 2 * N;
-  const size_t es = dtype_size(dtype);
-  char* basis = (char*)ws;
-  char* w = basis + (size_t)(m + 1) * fe * es;
-  auto Vk = [&](int k) { return (void*)(basis + (size_t)k * fe * es); };
-  char* sp = basis + L.basis;
-  GmState st;
-  st.H = carve<cx<double>>(sp, (size_t)N * (m + 1) * m);
-  st.cs = carve<cx<double>>(sp, (size_t)N * m);
-  st.sn = carve<cx<double>>(sp, (size_t)N * m);
-  st.g = carve<cx<double>>(sp, (size_t)N * (m + 1));
-  st.y = carve<double>(sp, (size_t)m * N * 2);
-  st.h1 = carve<double>(sp, (size_t)(m + 1) * N * 2);
-  st.h2 = carve<double>(sp, (size_t)(m + 1) * N * 2);
-  st.hn2 = carve<double>(sp, (size_t)N * 2);
-  st.beta2 = carve<double>(sp, (size_t)N * 2);
-  st.bnorm2 = carve<double>(sp, (size_t)N * 2);
-  st.inv = carve<double>(sp, (size_t)N);
-  st.conv = carve<int>(sp, N);
-  st.active = carve<int>(sp, N);
-  st.its = carve<int>(sp, N);
-  st.kend = carve<int>(sp, N);
-  st.counter = carve<int>(sp, 1);
-  double* part = (double*)(basis + L.basis + L.state);
-  int* hcount = c->hflag + 1;
-  auto read_counter = [&]() {
-    MRHS_CUDA(cudaMemcpyAsync(hcount, st.counter, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    MRHS_CUDA(cudaStreamSynchronize(c->stream));
-    return *hcount;
-  };
-  auto scale_into = [&](const void* x, void* y) {
-    MRHS_DISPATCH(dtype, S, (k_scale_rhs<S><<<grid_for(rows * N, 256), 256, 0, c->stream>>>((const S*)x, (S*)y, rows, N, st.inv)));
-    MRHS_LAUNCH_CHECK("scale_rhs");
-  };
-  MRHS_CUDA(cudaMemsetAsync(xc, 0, fe * es, c->stream));
-  multi_dot_ws(c, bc, 0, 1, bc, rows, N, dtype, st.bnorm2, part);
-  k_gm_init<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N);
-  MRHS_LAUNCH_CHECK("gm_init");
-  for (;;) {
-    apply_Dc(c, xc, w, N, dtype);
-    MRHS_DISPATCH(dtype, S, (k_sub_from<S><<<grid_for(fe, 256), 256, 0, c->stream>>>((const S*)bc, (S*)w, fe)));
-    MRHS_LAUNCH_CHECK("sub_from");
-    multi_dot_ws(c, w, 0, 1, w, rows, N, dtype, st.beta2, part);
-    MRHS_CUDA(cudaMemsetAsync(st.counter, 0, sizeof(int), c->stream));
-    k_gm_start<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N, m, tol, maxit);
-    MRHS_LAUNCH_CHECK("gm_start");
-    if (read_counter() == 0) break;
-    scale_into(w, Vk(0));
-    int kmax = 0;
-    for (int k = 0; k < m; ++k) {
-      apply_Dc(c, Vk(k), w, N, dtype);
-      multi_dot_ws(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, part, c->coef32);
-      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h1, -1.0, c->coef32);
-      multi_dot_ws(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, part, c->coef32);
-      multi_axpy(c, Vk(0), fe, k + 1, w, rows, N, dtype, st.h2, -1.0, c->coef32);
-      multi_dot_ws(c, w, 0, 1, w, rows, N, dtype, st.hn2, part);
-      MRHS_CUDA(cudaMemsetAsync(st.counter, 0, sizeof(int), c->stream));
-      k_gm_step<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N, m, k, tol, maxit);
-      MRHS_LAUNCH_CHECK("gm_step");
-      kmax = k + 1;
-      if (read_counter() == 0) break;
-      scale_into(w, Vk(k + 1));
-    }
-    k_gm_solve<<<grid_for(N, 64), 64, 0, c->stream>>>(st, N, m);
-    MRHS_LAUNCH_CHECK("gm_solve");
-    multi_axpy(c, Vk(0), fe, kmax, xc, rows, N, dtype, st.y, 1.0);
-  }
-  if (iters) {
-    MRHS_CUDA(cudaMemcpyAsync(iters, st.its, sizeof(int) * N, cudaMemcpyDeviceToHost, c->stream));
-    MRHS_CUDA(cudaStreamSynchronize(c->stream));
-  }
-  check_tc_timeout(c);
+  GmSpace sp;
+  sp.basis = (char*)ws;
+  sp.st = carve_state(sp.basis + L.basis, N, m);
+  sp.part = (double*)(sp.basis + L.basis + L.state);
+  coarse_gmres(c, bc, xc, N, dtype, tol, m, maxit, iters, (size_t)c->g.nagg * 2 * c->ntv, sp,
+               [&](const void* x, void* y) { apply_Dc(c, x, y, N, dtype); });
 }
 
 }  // namespace mrhs

@@ -216,7 +216,8 @@ struct mrhs_ctx_s {
 
   float* coef32 = nullptr;   // [65][256][2] float copy of BLAS coefficients
   int* dflag = nullptr;      // device error flag
-  int* hflag = nullptr;      // pinned host mirror
+  int* hflag = nullptr;      // pinned host mirror; words 8, 9: the coarse GMRES's convergence counts
+  cudaEvent_t gm_event[2] = {nullptr, nullptr};  // recorded after each count
   double* hbuf = nullptr;    // pinned host scratch
   size_t hbuf_bytes = 0;
 

@@ -696,6 +696,8 @@ void mrhs_destroy(mrhs_ctx c) {
   for (void* p : c->allocs) cudaFree(p);
   for (auto& b : c->scratch)
     if (b.p) cudaFree(b.p);
+  for (cudaEvent_t e : c->gm_event)
+    if (e) cudaEventDestroy(e);
   if (c->hflag) cudaFreeHost(c->hflag);
   if (c->hbuf) cudaFreeHost(c->hbuf);
   for (cudaEvent_t e : c->prof_events) cudaEventDestroy(e);
