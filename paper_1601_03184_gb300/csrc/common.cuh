@@ -189,6 +189,7 @@ struct mrhs_ctx_s {
   double* U64 = nullptr;  // [V][4][9] complex
   float* U32 = nullptr;
   float* U20 = nullptr;   // [V][4][20]: FP32 links padded to 80 bytes (float4-aligned records)
+  float* UQ = nullptr;    // [nagg][20][Va][4]: the same, sites innermost (float4 k of link mu at row 5 mu + k)
   double* A64 = nullptr;  // [V][2][36]
   float* A32 = nullptr;
   double* Ainv64 = nullptr;  // [V][2][36] inverse clover term (even-odd smoother), built on first use
@@ -258,6 +259,7 @@ enum Scratch {
   SC_EO1,         // even-odd domain solves: rho (even sites) / A^-1 H rho (odd sites)
   SC_EO2,         // q (even) and e (both parities), interleaved as two fields
   SC_COARSE_EO,   // even-odd coarse solve: two operator work fields and bhat
+  SC_TILES,       // tile copies of x and b for the on-chip smoother
   SC_COUNT
 };
 

@@ -151,22 +151,25 @@ __global__ void k_tables_canon(GeomArgs g, const int* nbr, const int* perm, cons
 // factor 1/2 and the antiperiodic sign of a hop across the t boundary belong
 // to the link (the forward hop from x and the backward hop from x+mu cross the
 // boundary together)
+// (UQ, may be null: the same, four floats of a link at a time and the sites of an
+// aggregate innermost: [aggregate][5 mu + k][Va] float4 with k < 5)
 __global__ void k_gauge_in(int s0, int ns, const int* perm, const double* Uc, double* U64, float* U32, float* U20,
-                           int Lt_last_start) {
+                           float* UQ, int Va, int Lt_last_start) {
   size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (t >= (size_t)ns * 80) return;
   size_t s = t / 80, e = t % 80;
   size_t sd = (size_t)perm[s0 + s];
   size_t mu = e / 20, k = e % 20;
+  float u20 = 0.f;
   if (k < 18) {
     double v = Uc[s * 72 + mu * 18 + k];
     U64[sd * 72 + mu * 18 + k] = v;
     U32[sd * 72 + mu * 18 + k] = (float)v;
     const bool flip = mu == 3 && (size_t)(s0 + s) >= (size_t)Lt_last_start;
-    U20[sd * 80 + e] = (float)(flip ? -0.5 * v : 0.5 * v);
-  } else {
-    U20[sd * 80 + e] = 0.f;
+    u20 = (float)(flip ? -0.5 * v : 0.5 * v);
   }
+  U20[sd * 80 + e] = u20;
+  if (UQ) UQ[((sd / Va * 20 + e / 4) * Va + sd % Va) * 4 + e % 4] = u20;
 }
 
 // ------------------------------------------------------------ clover ------
@@ -778,6 +781,8 @@ int mrhs_set_gauge(mrhs_ctx c, const double* U) {
       c->U64 = (double*)dalloc(c, n * sizeof(double));
       c->U32 = (float*)dalloc(c, n * sizeof(float));
       c->U20 = (float*)dalloc(c, (size_t)c->g.V * 80 * sizeof(float));
+      // 48^3 x 96: 3.4 GB, for the on-chip smoother of FP32 work fields
+      if (c->work_dtype == MRHS_F32 && c->g.Va > 128 && c->g.Va <= 256) c->UQ = (float*)dalloc(c, (size_t)c->g.V * 80 * sizeof(float));
     }
     // chunks of sites through the staging buffer bound the extra device memory
     const size_t per_site = 72 * sizeof(double);
@@ -788,7 +793,7 @@ int mrhs_set_gauge(mrhs_ctx c, const double* U) {
       MRHS_CUDA(cudaMemcpyAsync(st, U + s0 * 72, ns * per_site, cudaMemcpyHostToDevice, c->stream));
       const int lt_last = c->g.L[0] * c->g.L[1] * c->g.L[2] * (c->g.L[3] - 1);  // first canonical site with t = Lt-1
       k_gauge_in<<<grid_for((size_t)ns * 80, 256), 256, 0, c->stream>>>((int)s0, ns, c->perm, st, c->U64, c->U32, c->U20,
-                                                                       lt_last);
+                                                                       c->UQ, c->g.Va, lt_last);
       MRHS_LAUNCH_CHECK("gauge_in");
     }
     MRHS_CUDA(cudaStreamSynchronize(c->stream));
