@@ -69,11 +69,10 @@ struct Elem<tc::kFmtTF32> {
 
 using tc::tf32_split;
 
-// store the pair of elements (row, k), (row, k+1), k even, of a K-major tile
+// store a pair of K-adjacent elements at byte offset off of a K-major tile
 template <int FMT>
-__device__ __forceinline__ void put2(unsigned char* tile, int row, int k, float a, float b, int kg = kKG) {
+__device__ __forceinline__ void put2_at(unsigned char* tile, uint32_t off, float a, float b) {
   using E = Elem<FMT>;
-  const uint32_t off = tc::kmajor_offset(row, k, E::size, kg);
   if constexpr (E::size == 2) {
     *reinterpret_cast<uint32_t*>(tile + off) = E::pack(a, b);
   } else {
@@ -82,9 +81,7 @@ __device__ __forceinline__ void put2(unsigned char* tile, int row, int k, float 
 }
 
 // the same for split tf32: v = hi + lo, hi into one tile and lo into the other
-__device__ __forceinline__ void put2_split(unsigned char* thi, unsigned char* tlo, int row, int k, float a, float b,
-                                           int kg) {
-  const uint32_t off = tc::kmajor_offset(row, k, 4, kg);
+__device__ __forceinline__ void put2_split_at(unsigned char* thi, unsigned char* tlo, uint32_t off, float a, float b) {
   uint32_t ha, la, hb, lb;
   tf32_split(a, ha, la);
   tf32_split(b, hb, lb);
@@ -92,11 +89,198 @@ __device__ __forceinline__ void put2_split(unsigned char* thi, unsigned char* tl
   *reinterpret_cast<uint2*>(tlo + off) = make_uint2(la, lb);
 }
 
+// The links (and for k = 0 the clover term) of a chunk of sites, staged in shared
+// memory while the previous chunk is computed: per site the links of the eight hops
+// (5 float4 each: forward from the site, backward from the neighbour, those that
+// leave the aggregate skipped) and the two chirality blocks (18 float4)
+constexpr int kRecLinks = 40, kRec = 58;  // float4 of a site's record
+
+// the sites of block k in the order of their chunks (k = 0: all; k > 0: the face
+// x_mu = a_mu - 1, mu = k - 1): local index and coordinates
+struct AggSite {
+  int l, x[4];
+};
+__device__ __forceinline__ AggSite agg_site(const Agg4& g, int k, int f) {
+  AggSite r;
+  if (k == 0) {
+    r.l = f;
+  } else {
+    int S = 1;
+    for (int m = 0; m < k - 1; ++m) S *= g.a[m];
+    r.l = f % S + f / S * S * g.a[k - 1] + (g.a[k - 1] - 1) * S;
+  }
+  unsigned l = (unsigned)r.l;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    r.x[m] = (int)(l % (unsigned)g.a[m]);
+    l /= (unsigned)g.a[m];
+  }
+  return r;
+}
+// the same from a table in shared memory for blocks of at most kTabSites sites with
+// extents up to 256 (the divisions of agg_site are some 150 instructions a chunk)
+constexpr int kTabSites = 256;
+__device__ __forceinline__ AggSite tab_site(const uint32_t* tab, const Agg4& g, int k, int f) {
+  if (!tab) return agg_site(g, k, f);
+  const uint32_t t = tab[f];
+  AggSite r;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) r.x[m] = (int)(t >> (8 * m) & 255u);
+  r.l = r.x[0] + g.a[0] * (r.x[1] + g.a[1] * (r.x[2] + g.a[2] * r.x[3]));
+  return r;
+}
+
+__device__ __forceinline__ void cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
+
+// start the copies of the records of sites q0 .. q0 + nq - 1 of block k
+__device__ __forceinline__ void fetch_records(float4* rec, const float* __restrict__ U20, const float* __restrict__ Acl,
+                                              const Agg4& ag, const uint32_t* tab, int A, int Va, int k, int q0,
+                                              int nq) {
+  const int per = k == 0 ? kRec : 5;
+  for (int i = threadIdx.x; i < nq * per; i += kThreads) {
+    const int q = k == 0 ? i / kRec : i / 5, r = k == 0 ? i % kRec : i % 5;
+    const AggSite t = tab_site(tab, ag, k, q0 + q);
+    const size_t s = (size_t)A * Va + t.l;
+    if (k > 0) {
+      cp16(rec + q * kRec + 5 * (k - 1) + r, U20 + (s * 4 + k - 1) * 20 + 4 * r);
+      continue;
+    }
+    if (r < kRecLinks) {
+      const int d = r / 5, mu = d & 3;
+      size_t n = s;
+      if (d >= 4) {
+        const int S = mu == 0 ? 1 : mu == 1 ? ag.a[0] : mu == 2 ? ag.a[0] * ag.a[1] : ag.a[0] * ag.a[1] * ag.a[2];
+        const int xm = mu == 0 ? t.x[0] : mu == 1 ? t.x[1] : mu == 2 ? t.x[2] : t.x[3];
+        if (xm == 0) continue;
+        n = s - S;
+      }
+      cp16(rec + q * kRec + r, U20 + (n * 4 + mu) * 20 + 4 * (r - 5 * d));
+    } else {
+      cp16(rec + q * kRec + r, Acl + s * 72 + 4 * (r - kRecLinks));
+    }
+  }
+}
+
+// The column (hp, j) of Y = D_k P at a site: same[] the components of chirality hp,
+// other[] those of the other one; put_own takes the column of P itself there (the
+// chirality's six components). A hop acts on one spin s of the column: with
+// ch = U v_s (U^dag backward) and the chiral basis's B_mu,
+//   same_s -= ch,   other_t += phase ch,
+// t = 1 - s for mu = 0, 1 and s for mu = 2, 3, the phase +/- i for mu = 0, 2 and +/- 1
+// for mu = 1, 3. So one rolled loop over (spin, side) with signs as numbers serves
+// both chiralities, both sides and the faces; the spins swap names between the
+// passes. The size of the code matters here: with every hop instantiated by
+// itself the kernel ran at the rate of its instruction fetches (2.2 of 11 stalled
+// cycles per instruction; 2.5 to 2.9 ms at 16^3x32, ntv 32, whatever the number of
+// loads in flight or CTAs per SM). The next four neighbours' spin is loaded while
+// the present ones are computed.
+template <class SP, class PutOwn>
+__device__ __forceinline__ void dk_column(cx<float> same[6], cx<float> other[6], const SP* __restrict__ P,
+                                          const float4* rec, const AggSite& t, const Agg4& ag, int A, int B, int k,
+                                          int Va, int Nt, int j, int hp, PutOwn put_own) {
+  const size_t col0 = j + (size_t)12 * hp * Nt;
+  const SP* row0 = P + ((size_t)A * Va + t.l) * 24 * Nt + col0;
+  const int S1 = ag.a[0], S2 = S1 * ag.a[1], S3 = S2 * ag.a[2];
+  const int S[4] = {1, S1, S2, S3};
+  auto col = [&](const SP* row, int c) {
+    return mk<float>((float)to_r(row[(2 * c) * Nt]), (float)to_r(row[(2 * c + 1) * Nt]));
+  };
+  // the hops of pass (spin, side) that take part: inside the aggregate for k = 0, the
+  // one across the face for k > 0
+  auto on = [&](int mu, int side) {
+    return k == 0 ? (side == 0 ? t.x[mu] + 1 < ag.a[mu] : t.x[mu] > 0) : mu == k - 1;
+  };
+  cx<float> v[4][3], vn[4][3];
+  auto fetch = [&](int spin, int side) {
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu)
+      if (on(mu, side)) {
+        const SP* row = k == 0 ? row0 + (ptrdiff_t)(side == 0 ? S[mu] : -S[mu]) * 24 * Nt
+                               : P + ((size_t)B * Va + t.l - (ag.a[mu] - 1) * S[mu]) * 24 * Nt + col0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) vn[mu][c] = col(row + 6 * spin * Nt, c);
+      }
+  };
+  {
+    cx<float> own[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) own[c] = col(row0, c);
+    fetch(0, 0);
+    const float* q = reinterpret_cast<const float*>(rec + kRecLinks + 9 * hp);
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+      same[a] = other[a] = mk<float>(0, 0);
+      if (k == 0) {
+        // A is block diagonal in chirality: only block hp meets the column
+        cx<float> acc = scale(own[a], q[a]);
+#pragma unroll
+        for (int b = 0; b < 6; ++b) {
+          if (b == a) continue;
+          const int e = b > a ? herm_idx(a, b) : herm_idx(b, a);
+          const float2 m = *reinterpret_cast<const float2*>(q + e);
+          fma_(acc, mk(m.x, b > a ? m.y : -m.y), own[b]);
+        }
+        same[a] = acc;
+      }
+    }
+    put_own(own);
+  }
+  const float hs = hp ? -1.f : 1.f;
+  const int step = k == 0 ? 1 : 2;  // no backward side across a face
+#pragma unroll 1
+  for (int it = 0; it < 4; it += step) {
+    const int spin = it >> 1, side = it & 1;
+    const float sd = side ? -1.f : 1.f, ss = spin ? -1.f : 1.f;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) v[mu][c] = mk(vn[mu][c].re, sd * vn[mu][c].im);
+    if (it + step < 4) fetch((it + step) >> 1, (it + step) & 1);
+    // backward: U^dag v = conj(U^T conj(v)): v.im has been given the sign sd above
+    // and the imaginary part of the product gets it back where it is used
+    const float sg[4] = {hs * sd, -hs * ss * sd, hs * ss * sd, sd};
+    const int sa = side ? 2 : 6, sb = side ? 6 : 2;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+      if (!on(mu, side)) continue;
+      const float* u = reinterpret_cast<const float*>(rec + 5 * (4 * side + mu));
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        cx<float> ch = mk<float>(0, 0);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          const float2 l = *reinterpret_cast<const float2*>(u + a * sa + b * sb);
+          fma_(ch, mk(l.x, l.y), v[mu][b]);
+        }
+        same[a].re -= ch.re;
+        same[a].im = fmaf(-sd, ch.im, same[a].im);
+        cx<float>& o = other[(mu < 2 ? 3 : 0) + a];
+        if (mu & 1) {
+          o.re = fmaf(sg[mu], ch.re, o.re), o.im = fmaf(sg[mu] * sd, ch.im, o.im);
+        } else {
+          o.re = fmaf(-sg[mu] * sd, ch.im, o.re), o.im = fmaf(sg[mu], ch.re, o.im);
+        }
+      }
+    }
+    if (side == 1 || step == 2) {  // the other spin takes the first three places
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        cx<float> x = same[a];
+        same[a] = same[3 + a], same[3 + a] = x;
+        x = other[a];
+        other[a] = other[3 + a], other[3 + a] = x;
+      }
+    }
+  }
+}
+
 template <int FMT, class SP, bool SPLIT>
-__global__ void __launch_bounds__(kThreads) k_coarse_op_tc(const SP* __restrict__ P, const cx<float>* __restrict__ U,
-                                                           const float* __restrict__ Acl, const int* __restrict__ nbr,
-                                                           int Nt, Agg4 ag, int Va, cx<float>* __restrict__ Dc,
-                                                           int* __restrict__ err) {
+__global__ void __launch_bounds__(kThreads, 2) k_coarse_op_tc(const SP* __restrict__ P, const float* __restrict__ U20,
+                                                           const float* __restrict__ Acl,
+                                                           const int* __restrict__ aggnbr, int Nt, Agg4 ag, int Va,
+                                                           cx<float>* __restrict__ Dc, int* __restrict__ err) {
   constexpr int ES = Elem<FMT>::size;
   // 16-byte K groups per chunk: 12. Split tf32 keeps one stage of four tiles
   // (96 KB, two CTAs per SM): its chunk waits for the previous chunk's MMAs
@@ -113,18 +297,37 @@ __global__ void __launch_bounds__(kThreads) k_coarse_op_tc(const SP* __restrict_
   __shared__ uint32_t s_tmem;
   __shared__ int s_bad;
 
-  const int A = blockIdx.x / 5, k = blockIdx.x % 5;
+  // the self blocks first: they take several times as long as a forward block, and a
+  // last wave of them would leave most of the GPU idle (2.12 -> 1.79 ms with the
+  // cheaper operand offsets)
+  const int nagg = gridDim.x / 5;
+  const int A = (int)blockIdx.x < nagg ? blockIdx.x : (blockIdx.x - nagg) / 4;
+  const int k = (int)blockIdx.x < nagg ? 0 : 1 + (blockIdx.x - nagg) % 4;
   const int nc = 2 * Nt;
   const int NN = (2 * nc + 15) / 16 * 16;     // MMA N
   const int mu = k - 1;
   const int nsite = k == 0 ? Va : Va / ag.a[mu];
-  const int lmu = k == 0 ? 0 : ag.a[mu] - 1;
+  const int B = k == 0 ? A : aggnbr[A * 8 + mu];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int hp = threadIdx.x >> 7;  // the chirality of this warp's columns
 
   // zero both stages once: padding rows and off-chirality entries of A stay zero
   constexpr int NT = SPLIT ? 4 : 2;  // tiles per stage: A, B (and their low parts)
   for (int i = threadIdx.x; i < (ONE ? 1 : 2) * NT * TB / 16; i += kThreads)
     reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+  // the records of the chunks' sites, two chunks in turn
+  float4* rec = reinterpret_cast<float4*>(smem + (ONE ? 1 : 2) * NT * TB);
+  __shared__ uint32_t s_tab[kTabSites];
+  const bool small = nsite <= kTabSites && ag.a[0] <= 256 && ag.a[1] <= 256 && ag.a[2] <= 256 && ag.a[3] <= 256;
+  if (small)
+    for (int f = threadIdx.x; f < nsite; f += kThreads) {
+      const AggSite t = agg_site(ag, k, f);
+      s_tab[f] = t.x[0] | t.x[1] << 8 | t.x[2] << 16 | (unsigned)t.x[3] << 24;
+    }
+  __syncthreads();
+  const uint32_t* tab = small ? s_tab : nullptr;
+  fetch_records(rec, U20, Acl, ag, tab, A, Va, k, 0, min(Q, nsite));
+  asm volatile("cp.async.wait_all;" ::: "memory");
   if (threadIdx.x == 0) {
     tc::mbar_init(&mbar[0], 1);
     tc::mbar_init(&mbar[1], 1);
@@ -175,47 +378,51 @@ __global__ void __launch_bounds__(kThreads) k_coarse_op_tc(const SP* __restrict_
     unsigned char* tB = tA + TB;
     unsigned char* tAl = tA + 2 * TB;  // low parts (SPLIT)
     unsigned char* tBl = tA + 3 * TB;
-    // B: Y = D_k P for (site q, column col); absent sites of a ragged chunk give zeros
-    for (int w = threadIdx.x; w < Q * nc; w += kThreads) {
-      const int q = w / nc, col = w % nc;
-      cx<float> out[12];
+    if (t + 1 < nchunk)
+      fetch_records(rec + ((t + 1) & 1) * Q * kRec, U20, Acl, ag, tab, A, Va, k, q0 + Q, min(Q, nsite - q0 - Q));
+    // (site q, vector j) of the warp's chirality: B: Y = D_k P, A: P; absent sites
+    // of a ragged chunk give zeros
+    for (int w = threadIdx.x & 127; w < Q * Nt; w += 128) {
+      const int q = w / Nt, j = w - q * Nt;
+      const int col = hp * Nt + j;
+      // two components c, c + 1 of chirality h into rows (re, im) of a tile pair: byte
+      // offsets of the rows, then of the K index q * 12 + 6 h + c, c = 0, 2, 4
+      const uint32_t row_re = tc::kmajor_offset(col, 0, ES, KGT), row_im = tc::kmajor_offset(nc + col, 0, ES, KGT);
+      uint32_t ko[2][3];  // [same chirality, the other one]
 #pragma unroll
-      for (int c = 0; c < 12; ++c) out[c] = mk<float>(0, 0);
-      if (q < nq) {
-        const int l = k == 0 ? q0 + q : face_site(ag, mu, lmu, q0 + q);
-        const int s = A * Va + l;
-        if (col < Nt) dk_pcol<0, SP, float>(out, P, U, Acl, nbr, s, k, Nt, col, A * Va, Va);
-        else dk_pcol<1, SP, float>(out, P, U, Acl, nbr, s, k, Nt, col - Nt, A * Va, Va);
+      for (int i = 0; i < 3; ++i) {
+        ko[0][i] = tc::kmajor_offset(0, q * 12 + 6 * hp + 2 * i, ES, KGT);
+        ko[1][i] = tc::kmajor_offset(0, q * 12 + 6 * (1 - hp) + 2 * i, ES, KGT);
       }
-#pragma unroll
-      for (int c = 0; c < 12; c += 2) {
+      auto put = [&](unsigned char* hi, unsigned char* lo, uint32_t k2, cx<float> a, cx<float> b) {
         if constexpr (SPLIT) {
-          put2_split(tB, tBl, col, q * 12 + c, out[c].re, out[c + 1].re, KGT);
-          put2_split(tB, tBl, nc + col, q * 12 + c, out[c].im, out[c + 1].im, KGT);
+          put2_split_at(hi, lo, row_re + k2, a.re, b.re);
+          put2_split_at(hi, lo, row_im + k2, a.im, b.im);
         } else {
-          put2<FMT>(tB, col, q * 12 + c, out[c].re, out[c + 1].re);
-          put2<FMT>(tB, nc + col, q * 12 + c, out[c].im, out[c + 1].im);
+          put2_at<FMT>(hi, row_re + k2, a.re, b.re);
+          put2_at<FMT>(hi, row_im + k2, a.im, b.im);
         }
+      };
+      auto put_own = [&](const cx<float> own[6]) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) put(tA, tAl, ko[0][i], own[2 * i], own[2 * i + 1]);
+      };
+      cx<float> same[6], other[6];
+      if (q < nq) {
+        dk_column<SP>(same, other, P, rec + ((t & 1) * Q + q) * kRec, tab_site(tab, ag, k, q0 + q), ag, A, B, k, Va, Nt, j,
+                      hp, put_own);
+      } else {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) same[c] = other[c] = mk<float>(0, 0);
+        put_own(same);
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        put(tB, tBl, ko[0][i], same[2 * i], same[2 * i + 1]);
+        put(tB, tBl, ko[1][i], other[2 * i], other[2 * i + 1]);
       }
     }
-    // A: P rows (part p, h, j) for the components of chirality h
-    for (int w = threadIdx.x; w < nq * 12 * Nt; w += kThreads) {
-      const int j = w % Nt;
-      int rest = w / Nt;
-      const int p = rest % 2;
-      rest /= 2;
-      const int cp = rest % 3;
-      rest /= 3;
-      const int h = rest % 2;
-      const int q = rest / 2;
-      const int c = 6 * h + 2 * cp;
-      const int l = k == 0 ? q0 + q : face_site(ag, mu, lmu, q0 + q);
-      const size_t s = (size_t)A * Va + l;
-      const float a = to_r(P[((s * 12 + c) * 2 + p) * Nt + j]);
-      const float b = to_r(P[((s * 12 + c + 1) * 2 + p) * Nt + j]);
-      if constexpr (SPLIT) put2_split(tA, tAl, p * nc + h * Nt + j, q * 12 + c, a, b, KGT);
-      else put2<FMT>(tA, p * nc + h * Nt + j, q * 12 + c, a, b);
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     tc::fence_async_smem();
     // chunk t-1 done: fold its partial sum R into S before R is reused
     if (!ONE && t >= 1) {
@@ -566,8 +773,8 @@ bool build_Dc_tc(mrhs_ctx c, int fmt, bool split) {
   // two stages of 2 tiles, or one stage of 4 tiles (split; chunks of eight
   // sites in one stage of 196 KB per CTA measured slower: 270 against 184 ms
   // per build at 48^3x96)
-  const size_t smem = 4 * (size_t)kTileBytes;
-  const cx<float>* U = (const cx<float>*)c->U32;
+  const int chunk = split ? 4 : fmt == tc::kFmtTF32 ? 4 : 8;
+  const size_t smem = 4 * (size_t)kTileBytes + sizeof(float4) * 2 * chunk * kRec;
   const float* Acl = (const float*)c->A32;
   int* err = c->dflag + 2;
   MRHS_CUDA(cudaMemsetAsync(err, 0, sizeof(int), c->stream));
@@ -578,7 +785,7 @@ bool build_Dc_tc(mrhs_ctx c, int fmt, bool split) {
                 : split              ? k_coarse_op_tc<tc::kFmtTF32, SP, true>
                                      : k_coarse_op_tc<tc::kFmtTF32, SP, false>;
     MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    kern<<<c->g.nagg * 5, kThreads, smem, c->stream>>>((const SP*)c->P, U, Acl, c->nbr, Nt, ag, c->g.Va,
+    kern<<<c->g.nagg * 5, kThreads, smem, c->stream>>>((const SP*)c->P, c->U20, Acl, c->aggnbr, Nt, ag, c->g.Va,
                                                         (cx<float>*)c->Dc, err);
   });
   MRHS_LAUNCH_CHECK("coarse_op_tc");
