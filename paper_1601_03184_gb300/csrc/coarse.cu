@@ -299,47 +299,168 @@ __global__ void __launch_bounds__(256) k_restrict_tiled(const SP* __restrict__ P
   }
 }
 
-// FP32 restriction streamed through registers: one thread per (aggregate A,
-// chirality h, four rows i0..i0+3, four right-hand sides r0..r0+3), the sum
-// over the aggregate's sites and the chirality's six components in the
-// thread's registers (no staging, no barrier): every 16-byte load of P or v
-// feeds 16 complex products. Nt % 4 = 0, N % 4 = 0.
-__global__ void __launch_bounds__(128) k_restrict_stream(const float* __restrict__ P, const float* __restrict__ v,
-                                                         float* __restrict__ vc, int Nt, int N, int Va) {
-  const int A = blockIdx.x;
-  const int nq = N / 4, ni = Nt / 4;
-  const int t = threadIdx.x;
-  if (t >= 2 * ni * nq) return;
-  const int r0 = 4 * (t % nq), i0 = 4 * ((t / nq) % ni), h = t / (nq * ni);
-  float are[4][4], aim[4][4];
+// four consecutive values of a row in FP32
+template <class S>
+__device__ __forceinline__ void ld_four(const S* p, float v[4]) {
+  if constexpr (sizeof(S) == 4) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+  } else if constexpr (sizeof(S) == 2) {
+    const uint2 t = __ldg(reinterpret_cast<const uint2*>(p));
+    S h[4];
+    *reinterpret_cast<uint2*>(h) = t;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = to_r(h[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = (float)p[i];
+  }
+}
+
+// start the copy of the runs of n elements at site0 + i, i < ns, every `pitch`
+// elements, into consecutive shared memory (8-byte pieces: a run of 2-byte elements
+// starts on 8 bytes)
+template <class S>
+__device__ __forceinline__ void cp_runs(S* dst, const S* src, int n, size_t pitch, int ns) {
+  constexpr int E = 8 / (int)sizeof(S) > 0 ? 8 / (int)sizeof(S) : 1, W = sizeof(S) == 4 ? 4 : E;
+  const int per = n / W;  // pieces of a run (16 bytes for FP32)
+  for (int i = threadIdx.x; i < ns * per; i += 256) {
+    const int k = i / per, e = (i - k * per) * W;
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + k * n + e);
+    const S* p = src + k * pitch + e;
+    if constexpr (sizeof(S) == 4)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(p) : "memory");
+    else
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(p) : "memory");
+  }
+}
+// four consecutive values in shared memory in FP32
+template <class S>
+__device__ __forceinline__ void lds_four(const S* p, float v[4]) {
+  if constexpr (sizeof(S) == 4) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+  } else if constexpr (sizeof(S) == 2) {
+    const uint2 t = *reinterpret_cast<const uint2*>(p);
+    S h[4];
+    *reinterpret_cast<uint2*>(h) = t;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = to_r(h[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = (float)p[i];
+  }
+}
+
+// Restriction into FP32 coarse fields: one CTA per (aggregate A, chirality h); the
+// fine rows of kResSites sites of P and v are copied to shared memory one chunk ahead,
+// and a thread holds a tile of four coarse rows and NR right-hand sides and sums every
+// G-th fine row, G = 256 / tiles; the G sums of a tile are joined in shared memory in a
+// fixed order. Four 16-byte reads of shared memory feed 16 complex products, about the
+// balance of that pipe (4 cycles each) and the FMAs; the same reads from global memory
+// cost 16 to 20 cycles of the load unit each, cached or not. Per call, before (a thread
+// per tile over all rows, its reads from global memory) and after: FP32, 512
+// aggregates, 32 x 32: 913 -> 377 us; 20 x 20: 889 -> 205; 256, 8 x 8: 697 -> 59;
+// 256, 16 x 1: 493 -> 41; bf16, 8192, 24 x 24: 7392 -> 3987 us. VP, VV: 16-byte reads of
+// P (4 divides Nt) and of v (4 divides N, NR = 4).
+constexpr int kResSites = 8;
+template <class SP, class SV, int NR, bool VP, bool VV>
+__global__ void __launch_bounds__(256) k_restrict_split(const SP* __restrict__ P, const SV* __restrict__ v,
+                                                        float* __restrict__ vc, int Nt, int N, int Va) {
+  extern __shared__ double smem_d[];
+  // [2][kResSites][6][2][Nt] of P, then of v; the parts of the sums at the end
+  SP* sP = reinterpret_cast<SP*>(smem_d);
+  const int nP = 12 * Nt, nV = 12 * N;
+  SV* sV = reinterpret_cast<SV*>(smem_d + (2 * (size_t)kResSites * nP * sizeof(SP) + 15) / 16 * 2);
+  float2* part = reinterpret_cast<float2*>(smem_d);
+  const int A = blockIdx.x >> 1, h = blockIdx.x & 1;
+  const int nr = (N + NR - 1) / NR, ntile = (Nt + 3) / 4 * nr, G = 256 / ntile;
+  const int tile = threadIdx.x % ntile, g = threadIdx.x / ntile;
+  const int r0 = NR * (tile % nr), i0 = 4 * (tile / nr);
+  float are[4][NR], aim[4][NR];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) are[a][b] = aim[a][b] = 0.f;
-  const size_t row0 = (size_t)A * Va * 12 + 6 * h;
+    for (int b = 0; b < NR; ++b) are[a][b] = aim[a][b] = 0.f;
+  const SP* gP = P + ((size_t)A * Va * 2 + h) * nP;
+  const SV* gV = v + ((size_t)A * Va * 2 + h) * nV;
+  auto fetch = [&](int s0) {
+    const int ns = min(kResSites, Va - s0), buf = s0 / kResSites & 1;
+    cp_runs(sP + (size_t)buf * kResSites * nP, gP + (size_t)s0 * 2 * nP, nP, 2 * (size_t)nP, ns);
+    cp_runs(sV + (size_t)buf * kResSites * nV, gV + (size_t)s0 * 2 * nV, nV, 2 * (size_t)nV, ns);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  fetch(0);
+  for (int s0 = 0; s0 < Va; s0 += kResSites) {
+    const int nrow = 6 * min(kResSites, Va - s0), buf = s0 / kResSites & 1;
+    if (s0 + kResSites < Va) {
+      fetch(s0 + kResSites);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    const SP* bP = sP + (size_t)buf * kResSites * nP + i0;
+    const SV* bV = sV + (size_t)buf * kResSites * nV + r0;
+    if (g < G)
 #pragma unroll 2
-  for (int q = 0; q < Va * 6; ++q) {
-    const size_t row = row0 + (size_t)(q / 6) * 12 + q % 6;
-    const float4 pr = __ldg(reinterpret_cast<const float4*>(P + row * 2 * Nt + i0));
-    const float4 pi = __ldg(reinterpret_cast<const float4*>(P + (row * 2 + 1) * Nt + i0));
-    const float4 xr = __ldg(reinterpret_cast<const float4*>(v + row * 2 * N + r0));
-    const float4 xi = __ldg(reinterpret_cast<const float4*>(v + (row * 2 + 1) * N + r0));
-    const float Pr[4] = {pr.x, pr.y, pr.z, pr.w}, Pi[4] = {pi.x, pi.y, pi.z, pi.w};
-    const float Xr[4] = {xr.x, xr.y, xr.z, xr.w}, Xi[4] = {xi.x, xi.y, xi.z, xi.w};
+      for (int q = g; q < nrow; q += G) {
+        float pr[4], pi[4], xr[NR], xi[NR];
+        const SP* pp = bP + q * 2 * Nt;
+        const SV* pv = bV + q * 2 * N;
+        if constexpr (VP) {
+          lds_four(pp, pr), lds_four(pp + Nt, pi);
+        } else {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+          for (int a = 0; a < 4; ++a) {
+            const bool in = i0 + a < Nt;
+            pr[a] = in ? (float)to_r(pp[a]) : 0.f, pi[a] = in ? (float)to_r(pp[Nt + a]) : 0.f;
+          }
+        }
+        if constexpr (VV) {
+          lds_four(pv, xr), lds_four(pv + N, xi);
+        } else {
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        // conj(p) x: re = pr xr + pi xi, im = pr xi - pi xr
-        are[a][b] = fmaf(Pi[a], Xi[b], fmaf(Pr[a], Xr[b], are[a][b]));
-        aim[a][b] = fmaf(-Pi[a], Xr[b], fmaf(Pr[a], Xi[b], aim[a][b]));
+          for (int b = 0; b < NR; ++b) {
+            const bool in = r0 + b < N;
+            xr[b] = in ? (float)to_r(pv[b]) : 0.f, xi[b] = in ? (float)to_r(pv[N + b]) : 0.f;
+          }
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < NR; ++b) {
+            // conj(p) x: re = pr xr + pi xi, im = pr xi - pi xr
+            are[a][b] = fmaf(pi[a], xi[b], fmaf(pr[a], xr[b], are[a][b]));
+            aim[a][b] = fmaf(-pi[a], xr[b], fmaf(pr[a], xi[b], aim[a][b]));
+          }
       }
+    __syncthreads();  // the buffer takes the chunk after the next one
   }
+  // half of the tile entries at a time
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const size_t crow = (size_t)A * 2 * Nt + h * Nt + i0 + a;
-    *reinterpret_cast<float4*>(vc + fidx(crow, 0, N, r0)) = make_float4(are[a][0], are[a][1], are[a][2], are[a][3]);
-    *reinterpret_cast<float4*>(vc + fidx(crow, 1, N, r0)) = make_float4(aim[a][0], aim[a][1], aim[a][2], aim[a][3]);
+  for (int half = 0; half < 2; ++half) {
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < NR; ++b)
+        part[(a * NR + b) * 256 + threadIdx.x] = make_float2(are[2 * half + a][b], aim[2 * half + a][b]);
+    __syncthreads();
+    for (int e = threadIdx.x; e < 2 * NR * ntile; e += 256) {
+      const int t = e % ntile, ab = e / ntile;
+      float2 s = make_float2(0.f, 0.f);
+      for (int k = 0; k < G; ++k) {
+        const float2 o = part[ab * 256 + k * ntile + t];
+        s.x += o.x, s.y += o.y;
+      }
+      const int i = 4 * (t / nr) + 2 * half + ab / NR, r = NR * (t % nr) + ab % NR;
+      if (i < Nt && r < N) {
+        const size_t crow = ((size_t)A * 2 + h) * Nt + i;
+        vc[fidx(crow, 0, N, r)] = s.x;
+        vc[fidx(crow, 1, N, r)] = s.y;
+      }
+    }
   }
 }
 
@@ -541,48 +662,99 @@ __global__ void k_prolong6(const SP* __restrict__ P, const SC* __restrict__ uc, 
   for (int cc = 0; cc < 6; ++cc) st<SU, R>(u, s * 12 + 6 * h + cc, N, r, acc[cc]);
 }
 
-// The same for FP32 coarse and fine fields with N % 4 == 0: four right-hand
-// sides per thread (16-byte loads of uc and stores of u), so every P entry
-// loaded serves 4 x 6 complex products; the scalar kernel's operations in
-// its order (the same bits).
+// The same for FP32 fields with N % 4 == 0 and Nt % 4 == 0: per (aggregate, chirality)
+// the product of the 6 Va x Nt rows of P with the Nt x N coarse block, which is staged
+// in shared memory; a thread holds four fine rows and four right-hand sides, and reads
+// four columns j of its rows of P at once: sixteen 16-byte reads feed 256 FMAs, where one
+// site's six rows and a single column per step took fourteen reads for 96. The sums
+// run over j in order, as in the other forms. Per call, before and after: 512
+// aggregates, 32 x 32, FP32: 514 -> 326 us; 8192, 24 x 24, bf16 P: 4822 -> 3112 us.
+constexpr int kProRows = 4;
 template <class SP>
-__global__ void k_prolong6x4(const SP* __restrict__ P, const float* __restrict__ uc, float* __restrict__ u, int Nt,
-                             int N, int Va, size_t nwork) {
-  const int Q = N / 4;
+__global__ void __launch_bounds__(256) k_prolong_tile(const SP* __restrict__ P, const float* __restrict__ uc,
+                                                      float* __restrict__ u, int Nt, int N, int Va) {
+  extern __shared__ double smem_d[];
+  float4* w = reinterpret_cast<float4*>(smem_d);  // [Nt][2][N / 4]
+  const int A = blockIdx.x >> 1, h = blockIdx.x & 1, Q = N / 4;
+  const float4* src = reinterpret_cast<const float4*>(uc + ((size_t)A * 2 + h) * Nt * 2 * N);
+  for (int i = threadIdx.x; i < Nt * 2 * Q; i += 256) w[i] = __ldg(src + i);
+  __syncthreads();
+  const int nrow = 6 * Va, ng = (nrow + kProRows - 1) / kProRows;
+  for (int t = blockIdx.y * 256 + threadIdx.x; t < ng * Q; t += gridDim.y * 256) {
+    const int q = t % Q, l0 = t / Q * kProRows;
+    size_t row[kProRows];
+#pragma unroll
+    for (int a = 0; a < kProRows; ++a) {
+      const int l = min(l0 + a, nrow - 1);
+      row[a] = ((size_t)A * Va + l / 6) * 12 + 6 * h + l % 6;
+    }
+    float are[kProRows][4], aim[kProRows][4];
+#pragma unroll
+    for (int a = 0; a < kProRows; ++a)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) are[a][e] = aim[a][e] = 0.f;
+    for (int j = 0; j < Nt; j += 4) {
+      float pr[kProRows][4], pi[kProRows][4];
+#pragma unroll
+      for (int a = 0; a < kProRows; ++a) {
+        ld_four(P + row[a] * 2 * Nt + j, pr[a]);
+        ld_four(P + row[a] * 2 * Nt + Nt + j, pi[a]);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 w0 = w[(j + i) * 2 * Q + q], w1 = w[((j + i) * 2 + 1) * Q + q];
+        const float wr[4] = {w0.x, w0.y, w0.z, w0.w}, wi[4] = {w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+        for (int a = 0; a < kProRows; ++a)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            are[a][e] = fmaf(-pi[a][i], wi[e], fmaf(pr[a][i], wr[e], are[a][e]));
+            aim[a][e] = fmaf(pi[a][i], wr[e], fmaf(pr[a][i], wi[e], aim[a][e]));
+          }
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < kProRows; ++a)
+      if (l0 + a < nrow) {
+        *reinterpret_cast<float4*>(u + fidx(row[a], 0, N, 4 * q)) = make_float4(are[a][0], are[a][1], are[a][2], are[a][3]);
+        *reinterpret_cast<float4*>(u + fidx(row[a], 1, N, 4 * q)) = make_float4(aim[a][0], aim[a][1], aim[a][2], aim[a][3]);
+      }
+  }
+}
+
+// One right-hand side, FP32 fields, Nt % 4 == 0 (the V-cycle of a solve): LPR
+// neighbouring lanes share a fine row, four columns of P each at a time, and join
+// their sums by shuffles; P is read once in full lines (16 vectors, 65536 sites,
+// 100 MB: 116 -> 27 us; a thread per (site, chirality) read 4 bytes of each row at
+// a time).
+template <class SP, int LPR>
+__global__ void __launch_bounds__(256) k_prolong_one(const SP* __restrict__ P, const float* __restrict__ uc,
+                                                     float* __restrict__ u, int Nt, int Va, size_t nrow) {
   const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (t >= nwork) return;
-  const int r0 = 4 * (int)(t % Q);
-  const size_t q = t / Q;
-  const int h = (int)(q % 2);
-  const size_t s = q / 2;
-  const size_t A = s / Va;
-  float are[6][4], aim[6][4];
+  const int lane = (int)(t % LPR);
+  const size_t row = t / LPR;  // site * 12 + c
+  float re = 0.f, im = 0.f;
+  if (row < nrow) {
+    const size_t A = row / 12 / Va;
+    const float* w = uc + (A * 2 + (row % 12) / 6) * Nt * 2;
+    for (int j = 4 * lane; j < Nt; j += 4 * LPR) {
+      float pr[4], pi[4];
+      ld_four(P + row * 2 * Nt + j, pr);
+      ld_four(P + row * 2 * Nt + Nt + j, pi);
 #pragma unroll
-  for (int cc = 0; cc < 6; ++cc)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) are[cc][e] = aim[cc][e] = 0.f;
-  for (int j = 0; j < Nt; ++j) {
-    const size_t crow = A * 2 * Nt + h * Nt + j;
-    const float4 w0 = *reinterpret_cast<const float4*>(uc + fidx(crow, 0, N, r0));
-    const float4 w1 = *reinterpret_cast<const float4*>(uc + fidx(crow, 1, N, r0));
-    const float wr[4] = {w0.x, w0.y, w0.z, w0.w}, wi[4] = {w1.x, w1.y, w1.z, w1.w};
-#pragma unroll
-    for (int cc = 0; cc < 6; ++cc) {
-      const cx<float> pv = ld<SP, float>(P, s * 12 + 6 * h + cc, Nt, j);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        // fma_(acc, p, w): acc.re += p.re w.re - p.im w.im, acc.im += p.re w.im + p.im w.re
-        are[cc][e] = fmaf(-pv.im, wi[e], fmaf(pv.re, wr[e], are[cc][e]));
-        aim[cc][e] = fmaf(pv.im, wr[e], fmaf(pv.re, wi[e], aim[cc][e]));
+      for (int i = 0; i < 4; ++i) {
+        const float2 v = __ldg(reinterpret_cast<const float2*>(w) + j + i);
+        re = fmaf(-pi[i], v.y, fmaf(pr[i], v.x, re));
+        im = fmaf(pi[i], v.x, fmaf(pr[i], v.y, im));
       }
     }
   }
 #pragma unroll
-  for (int cc = 0; cc < 6; ++cc) {
-    const size_t row = s * 12 + 6 * h + cc;
-    *reinterpret_cast<float4*>(u + fidx(row, 0, N, r0)) = make_float4(are[cc][0], are[cc][1], are[cc][2], are[cc][3]);
-    *reinterpret_cast<float4*>(u + fidx(row, 1, N, r0)) = make_float4(aim[cc][0], aim[cc][1], aim[cc][2], aim[cc][3]);
+  for (int o = LPR / 2; o >= 1; o >>= 1) {
+    re += __shfl_xor_sync(0xffffffffu, re, o);
+    im += __shfl_xor_sync(0xffffffffu, im, o);
   }
+  if (lane == 0 && row < nrow) *reinterpret_cast<float2*>(u + 2 * row) = make_float2(re, im);
 }
 
 template <class S>
@@ -847,15 +1019,24 @@ void restrict_typed(mrhs_ctx c, const void* v, int dv, void* vc, int dc, int N) 
   MRHS_REQUIRE(threads <= 1024, MRHS_ERR_SHAPE, "restriction: ntv*nrhs too large");
   MRHS_REQUIRE(dc == MRHS_F64 || dc == MRHS_F32, MRHS_ERR_ARG, "coarse fields are F64 or F32");
   Prof pr(c, "restrict");
-  static const bool stream_off = [] {
+  static const bool split_off = [] {
     const char* e = std::getenv("MRHS_RESTRICT");
     return e && std::string(e) == "tiled";
   }();
-  if (!stream_off && c->tv_dtype == MRHS_F32 && dv == MRHS_F32 && dc == MRHS_F32 && Nt % 4 == 0 && N % 4 == 0 &&
-      2 * (Nt / 4) * (N / 4) <= 128) {
-    k_restrict_stream<<<c->g.nagg, 128, 0, c->stream>>>((const float*)c->P, (const float*)v, (float*)vc, Nt, N,
-                                                        c->g.Va);
-    MRHS_LAUNCH_CHECK("restrict_stream");
+  if (!split_off && dc == MRHS_F32) {
+    const bool vp = Nt % 4 == 0, vv = N % 4 == 0;
+    MRHS_DISPATCH(c->tv_dtype, SP, MRHS_DISPATCH(dv, SV, {
+      auto kern = N <= 3 && vp ? k_restrict_split<SP, SV, 1, true, false>
+                  : N <= 3     ? k_restrict_split<SP, SV, 1, false, false>
+                  : vp && vv   ? k_restrict_split<SP, SV, 4, true, true>
+                               : k_restrict_split<SP, SV, 4, false, false>;
+      const size_t stage = 2 * (size_t)kResSites * 12;
+      const size_t smem = std::max((stage * Nt * sizeof(SP) + 15) / 16 * 16 + stage * N * sizeof(SV),
+                                   sizeof(float2) * 256 * 2 * (N <= 3 ? 1 : 4));
+      MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      kern<<<2 * c->g.nagg, 256, smem, c->stream>>>((const SP*)c->P, (const SV*)v, (float*)vc, Nt, N, c->g.Va);
+    }));
+    MRHS_LAUNCH_CHECK("restrict_split");
     return;
   }
   const bool tiled = Nt % 4 == 0 && N % 2 == 0 && (nc / 4) * (N / 2) <= 256;
@@ -892,10 +1073,24 @@ void prolong_typed(mrhs_ctx c, const void* uc, int dc, void* u, int du, int N) {
   MRHS_REQUIRE(dc == MRHS_F64 || dc == MRHS_F32, MRHS_ERR_ARG, "coarse fields are F64 or F32");
   size_t work = (size_t)c->g.V * 2 * N;
   Prof pr(c, "prolong");
-  if (dc == MRHS_F32 && du == MRHS_F32 && N % 4 == 0 && ((uintptr_t)uc & 15) == 0 && ((uintptr_t)u & 15) == 0) {
-    const size_t w4 = (size_t)c->g.V * 2 * (N / 4);
-    MRHS_DISPATCH(c->tv_dtype, SP, (k_prolong6x4<SP><<<grid_for(w4, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, w4)));
-    MRHS_LAUNCH_CHECK("prolong");
+  const bool aligned = ((uintptr_t)uc & 15) == 0 && ((uintptr_t)u & 15) == 0;
+  const size_t smem = sizeof(float) * 2 * (size_t)c->ntv * N;
+  if (dc == MRHS_F32 && du == MRHS_F32 && c->ntv % 4 == 0 && N % 4 == 0 && aligned && smem <= 48 * 1024) {
+    // (two rounds of a CTA's threads over its rows: the coarse block staged serves them)
+    const dim3 grid(2 * c->g.nagg, std::max(1, 6 * c->g.Va / kProRows * (N / 4) / 512));
+    MRHS_DISPATCH(c->tv_dtype, SP, (k_prolong_tile<SP><<<grid, 256, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va)));
+    MRHS_LAUNCH_CHECK("prolong_tile");
+    return;
+  }
+  if (dc == MRHS_F32 && du == MRHS_F32 && c->ntv % 4 == 0 && N == 1 && aligned) {
+    const size_t nrow = (size_t)c->g.V * 12;
+    MRHS_DISPATCH(c->tv_dtype, SP, {
+      if (c->ntv <= 16)
+        k_prolong_one<SP, 4><<<grid_for(nrow * 4, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, c->g.Va, nrow);
+      else
+        k_prolong_one<SP, 8><<<grid_for(nrow * 8, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, c->g.Va, nrow);
+    });
+    MRHS_LAUNCH_CHECK("prolong_one");
     return;
   }
   MRHS_DISPATCH(c->tv_dtype, SP, MRHS_DISPATCH(du, SU, {
