@@ -226,86 +226,169 @@ __global__ void k_modrelu_back(const float* z, const float* dh, float* dz, const
   }
 }
 
-// weight gradient partials: CTA (k, site range); thread (c, c') pairs over
-// the CTA's sites and all right-hand sides; one right-hand side and 8 sites
-// staged at a time
-constexpr int kWgSites = 8;
-__global__ void k_wgrad(const float* __restrict__ dz, const float* __restrict__ h, const float* __restrict__ U32,
-                        const int* __restrict__ nbr, int cin, int cout, int N, size_t V, size_t sites_per_cta,
-                        double* part) {
-  __shared__ cx<float> sdz[kWgSites][kMaxC][3];
-  __shared__ cx<float> stv[kWgSites][kMaxC][3];
-  const int k = blockIdx.y;
-  const size_t s0 = blockIdx.x * sites_per_cta;
+// Weight gradient partials: G[k][c][c'] = sum over (site, colour, right-hand side) m
+// of dz[m][c] conj(t_k[m][c']), t_k the transported input of step k. CTA (k, range of
+// sites); tiles of sites x NB right-hand sides (cols columns, M = 3 cols with the colours)
+// of dz and t_k are staged in shared memory, and a thread holds 4 x 4 entries (c, c')
+// and every G-th m, G = 256 / (4 x 4 tiles): eight 8-byte reads feed 64 FMAs, about
+// the balance of the two pipes. The FP32 sums run over at most kWgChain m and are
+// then added into (hi, lo) pairs (two-sum, 48 bits), FP64 being 1/64 of the FP32
+// rate here; the pairs of a tile's threads are joined in FP64 at the end.
+// Before, a CTA staged 8 sites of one right-hand side at a time and each thread took
+// one (c, c') with two 8-byte reads and 3 FMAs per read: 2461 us a layer on average at
+// 16^4 sites, 8 right-hand sides, widths 4-11-11-4; now 1174 us (the loads of a tile in
+// turn, then the joins at the end, are what is left).
+constexpr int kWgChain = 32;
+
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+  hi = s;
+}
+
+__global__ void __launch_bounds__(256, 2) k_wgrad(const float* __restrict__ dz, const float* __restrict__ h,
+                                               const float* __restrict__ U32, const int* __restrict__ nbr, int cin,
+                                               int cout, int N, size_t V, size_t sites_per_cta, int cols,
+                                               double* part) {
+  const int M = 3 * cols;
+  extern __shared__ double smem_wg[];
+  float2* sdz = reinterpret_cast<float2*>(smem_wg);  // [4 ceil(cout/4)][M], the rows beyond cout zero
+  const int nci = (cin + 3) / 4, nco = (cout + 3) / 4, ntile = nci * nco, G = 256 / ntile;
+  float2* stv = sdz + 4 * nco * M;                // [4 ceil(cin/4)][M]
+  const int k = blockIdx.x, tid = threadIdx.x;
+  const size_t s0 = blockIdx.y * sites_per_cta;
   const size_t s1 = min(V, s0 + sites_per_cta);
-  const int npair = cout * cin;
-  double accr[4] = {0, 0, 0, 0}, acci[4] = {0, 0, 0, 0};
-  for (size_t sb = s0; sb < s1; sb += kWgSites) {
-    const int ns = (int)min((size_t)kWgSites, s1 - sb);
-    for (int r = 0; r < N; ++r) {
-      for (int w = threadIdx.x; w < ns * cout * 3; w += blockDim.x) {
-        const int q = w / (cout * 3), c = (w / 3) % cout, a = w % 3;
-        const size_t row = ((sb + q) * cout + c) * 3 + a;
-        sdz[q][c][a] = mk(dz[fidx(row, 0, N, r)], dz[fidx(row, 1, N, r)]);
-      }
-      for (int w = threadIdx.x; w < ns * cin; w += blockDim.x) {
-        const int q = w / cin, cp = w % cin;
+  const int NB = min(N, 8), SB = cols / NB;       // right-hand sides and sites of a tile
+  const int LC = 32 / NB, lr = (tid & 31) < LC * NB ? (tid & 31) % NB : NB, lc = (tid & 31) / NB;  // staging lanes
+  const int g = tid % G, tile = tid / G;             // neighbouring lanes: neighbouring m
+  const bool on = tile < ntile;
+  const int c0 = 4 * (tile / nci), d0 = 4 * (tile % nci);
+  float acc[32], hi[32], lo[32];                     // [4][4][re, im]
+#pragma unroll
+  for (int e = 0; e < 32; ++e) acc[e] = hi[e] = lo[e] = 0.f;
+  for (int i = tid; i < 4 * (nco + nci) * M; i += 256) sdz[i] = make_float2(0.f, 0.f);
+  __syncthreads();
+  int chain = 0;
+  for (size_t sb = s0; sb < s1; sb += SB) {
+    const int ns = (int)min((size_t)SB, s1 - sb);
+    for (int r0 = 0; r0 < N; r0 += NB) {
+      const int nr = min(NB, N - r0), mm = 3 * ns * nr;
+      // a warp takes a site: lanes (right-hand side, channel), the link and the
+      // neighbour of the step once for all channels
+#pragma unroll 2
+      for (int q = tid >> 5; q < ns; q += 8) {
+        const size_t x = sb + q;
         cx<float> T[3][3];
         size_t n;
         float sg;
-        link_k(T, U32, nbr, sb + q, k, n, sg);
-        cx<float> hv[3];
+        link_k(T, U32, nbr, x, k, n, sg);
+        if (lr < nr) {
+          for (int c = lc; c < cout; c += LC) {
+            const float* p = dz + fidx((x * cout + c) * 3, 0, N, r0 + lr);
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-          const size_t row = (n * cin + cp) * 3 + b;
-          hv[b] = mk(h[fidx(row, 0, N, r)], h[fidx(row, 1, N, r)]);
-        }
+            for (int a = 0; a < 3; ++a)
+              sdz[c * M + (a * ns + q) * nr + lr] = make_float2(p[(2 * a) * N], p[(2 * a + 1) * N]);
+          }
+          for (int c = lc; c < cin; c += LC) {
+            const float* p = h + fidx((n * cin + c) * 3, 0, N, r0 + lr);
+            cx<float> hv[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-          cx<float> s = mk(0.f, 0.f);
+            for (int b = 0; b < 3; ++b) hv[b] = mk(sg * p[(2 * b) * N], sg * p[(2 * b + 1) * N]);
 #pragma unroll
-          for (int b = 0; b < 3; ++b) fma_(s, T[a][b], hv[b]);
-          stv[q][cp][a] = scale(s, sg);
+            for (int a = 0; a < 3; ++a) {
+              cx<float> s = mk(0.f, 0.f);
+#pragma unroll
+              for (int b = 0; b < 3; ++b) fma_(s, T[a][b], hv[b]);
+              stv[c * M + (a * ns + q) * nr + lr] = make_float2(s.re, s.im);
+            }
+          }
         }
       }
       __syncthreads();
+      if (on) {
+        for (int m = g; m < mm; m += G) {
+          float2 z[4], t[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int p = threadIdx.x + e * blockDim.x;
-        if (p >= npair) break;
-        const int c = p / cin, cp = p % cin;
-        cx<float> s = mk(0.f, 0.f);
-        for (int q = 0; q < ns; ++q)
+          for (int i = 0; i < 4; ++i) z[i] = sdz[(c0 + i) * M + m], t[i] = stv[(d0 + i) * M + m];
 #pragma unroll
-          for (int a = 0; a < 3; ++a) fmac_(s, stv[q][cp][a], sdz[q][c][a]);  // dz conj(t)
-        accr[e] += s.re;
-        acci[e] += s.im;
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              float& re = acc[(4 * i + j) * 2];
+              float& im = acc[(4 * i + j) * 2 + 1];
+              // dz conj(t)
+              re = fmaf(z[i].x, t[j].x, fmaf(z[i].y, t[j].y, re));
+              im = fmaf(z[i].y, t[j].x, fmaf(-z[i].x, t[j].y, im));
+            }
+        }
+        chain += (mm + G - 1) / G;
+        if (chain + (M + G - 1) / G > kWgChain) {
+#pragma unroll
+          for (int e = 0; e < 32; ++e) two_sum(hi[e], lo[e], acc[e]), acc[e] = 0.f;
+          chain = 0;
+        }
       }
       __syncthreads();
     }
   }
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const int p = threadIdx.x + e * blockDim.x;
-    if (p >= npair) break;
-    double* o = part + (((size_t)k * gridDim.x + blockIdx.x) * npair + p) * 2;
-    o[0] = accr[e];
-    o[1] = acci[e];
+  for (int e = 0; e < 32; ++e) two_sum(hi[e], lo[e], acc[e]);
+  // the G threads of a tile, eight entries at a time: four neighbouring threads sum a
+  // quarter of them each and join by shuffles (a fixed order)
+  double2* sum = reinterpret_cast<double2*>(smem_wg);  // [8][256]
+  const int npair = cout * cin;
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int i = 8 * half + e;
+      sum[e * 256 + tid] =
+          make_double2((double)hi[2 * i] + (double)lo[2 * i], (double)hi[2 * i + 1] + (double)lo[2 * i + 1]);
+    }
+    __syncthreads();
+    for (int w = tid; w < ntile * 32; w += 256) {  // a warp per tile
+      const int quarter = w & 3, e = w >> 2 & 7, tl = w >> 5;
+      double2 s = make_double2(0, 0);
+      for (int i = quarter; i < G; i += 4) {
+        const double2 v = sum[e * 256 + tl * G + i];
+        s.x += v.x, s.y += v.y;
+      }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+      }
+      const int i = 8 * half + e, c = 4 * (tl / nci) + i / 4, cp = 4 * (tl % nci) + i % 4;
+      if (quarter == 0 && c < cout && cp < cin) {
+        double* o = part + (((size_t)k * gridDim.y + blockIdx.y) * npair + c * cin + cp) * 2;
+        o[0] = s.x;
+        o[1] = s.y;
+      }
+    }
   }
 }
 
-// G[k][p] += factor * sum of the per-CTA partials (fixed order)
+// G[k][p] += factor * sum of the per-CTA partials: a warp per (k, p), its lanes the
+// chunks l, l + 32, ..., joined by a fixed butterfly
 __global__ void k_wgrad_sum(const double* part, int nchunk, int npair, float* G, float factor) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (t >= 9 * npair) return;
   const int k = t / npair, p = t % npair;
   double a = 0, b = 0;
-  for (int ch = 0; ch < nchunk; ++ch) {
-    a += part[(((size_t)k * nchunk + ch) * npair + p) * 2];
-    b += part[(((size_t)k * nchunk + ch) * npair + p) * 2 + 1];
+  for (int ch = lane; ch < nchunk; ch += 32) {
+    const double2 v = *reinterpret_cast<const double2*>(part + (((size_t)k * nchunk + ch) * npair + p) * 2);
+    a += v.x, b += v.y;
   }
-  G[2 * t] += (float)(factor * a);
-  G[2 * t + 1] += (float)(factor * b);
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  if (lane == 0) {
+    G[2 * t] += (float)(factor * a);
+    G[2 * t + 1] += (float)(factor * b);
+  }
 }
 
 __global__ void k_bias_sum(const double* part, int nchunk, int C, float* G) {
@@ -430,16 +513,23 @@ void nn_forward_impl(mrhs_ctx c, const float* in, float* out, int N) {
 void wgrad(mrhs_ctx c, NNState& s, const float* dz, const float* h, int l, int N) {
   const int cin = s.C[l], cout = s.C[l + 1];
   const size_t V = c->g.V;
-  const int nchunk = (int)std::min<size_t>(256, (V + 511) / 512);
+  // ranges of sites: nine CTAs (the steps) each; the buffer holds 256
+  const int nchunk = (int)std::min<size_t>(256, (V + 255) / 256);
   const size_t per = (V + nchunk - 1) / nchunk;
   const size_t need = (size_t)9 * nchunk * cout * cin * 2;
   MRHS_REQUIRE(need <= s.part_elems, MRHS_ERR_ARG, "nn: partial buffer too small");
-  dim3 grid(nchunk, 9);
+  // 128 columns a tile where two CTAs of it fit on an SM (a tile waits for its loads
+  // once or twice, whatever its size), else 64
+  const size_t per_col = sizeof(float2) * 3 * 4 * ((cout + 3) / 4 + (cin + 3) / 4);
+  const int cols = per_col * 128 <= 100 * 1024 ? 128 : 64;
+  const size_t smem = std::max(per_col * cols, sizeof(double2) * 256 * 8);
+  MRHS_CUDA(cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   Prof pr(c, "nn_wgrad");
-  k_wgrad<<<grid, 256, 0, c->stream>>>(dz, h, c->U32, c->nbr, cin, cout, N, V, per, s.part);
+  // the steps fastest, so that the nine CTAs of a range share its dz and h in L2
+  k_wgrad<<<dim3(9, nchunk), 256, smem, c->stream>>>(dz, h, c->U32, c->nbr, cin, cout, N, V, per, cols, s.part);
   MRHS_LAUNCH_CHECK("wgrad");
-  k_wgrad_sum<<<grid_for((size_t)9 * cout * cin, 256), 256, 0, c->stream>>>(s.part, nchunk, cout * cin,
-                                                                            s.G + 2 * layer_off(s, l), 1.f);
+  k_wgrad_sum<<<grid_for((size_t)9 * cout * cin * 32, 256), 256, 0, c->stream>>>(s.part, nchunk, cout * cin,
+                                                                                 s.G + 2 * layer_off(s, l), 1.f);
   MRHS_LAUNCH_CHECK("wgrad_sum");
 }
 
