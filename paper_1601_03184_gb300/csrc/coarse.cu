@@ -1126,8 +1126,9 @@ void apply_Dc_part(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, int dtype) 
     const char* e = std::getenv("MRHS_DC_APPLY");
     return e && std::string(e) == "alu";
   }();
-  if (c->dc_engine != MRHS_DC_ALU && dtype == MRHS_F32 && !apply_alu) {
-    const bool split = c->prec == MRHS_PREC_FP32;
+  // (the mixed setups' other counts of right-hand sides keep FP32 accuracy: split)
+  if (c->dc_engine != MRHS_DC_ALU && dtype == MRHS_F32 && !apply_alu && nrhs > kRowsMaxRhs) {
+    const bool split = c->prec == MRHS_PREC_FP32 || nrhs % 16 != 0;
     if (apply_Dc_tc(c, pt, yc, nrhs, split)) return;
   }
   Prof pr(c, "apply_dc");

@@ -530,7 +530,8 @@ __global__ void __launch_bounds__(kDcThreads, 1) k_apply_dc_tc(const float* __re
   __shared__ int s_bad;
   const int A = alist ? alist[blockIdx.x] : (int)blockIdx.x;
   const int nk = ke - kb;                    // blocks of this launch (at least 1)
-  const int NM = 2 * nrhs;                   // MMA N
+  const int NX = 2 * nrhs;                   // columns: Re, Im of the right-hand sides
+  const int NM = (NX + 15) & ~15;            // MMA N (the columns beyond NX are zero)
   const int KG = nc / 4;                     // 16-byte K groups (tf32)
   const int a_bytes = kRows / 8 * KG * 128;  // A tile
   const int b_bytes = NM / 8 * KG * 128;     // B tile
@@ -550,6 +551,13 @@ __global__ void __launch_bounds__(kDcThreads, 1) k_apply_dc_tc(const float* __re
   if (!PRE && 2 * nc < kRows) {  // rows of A beyond 2nc stay zero
     const int nz = (SPLIT ? 2 : 1) * (a_bytes + b_bytes) / 16;
     for (int i = tid; i < nz; i += kDcThreads) reinterpret_cast<uint4*>(Ahi)[i] = make_uint4(0, 0, 0, 0);
+  }
+  if (NM > NX) {  // so do the columns of B beyond the right-hand sides
+    for (int u = tid; u < (NM - NX) * KG; u += kDcThreads) {
+      const uint32_t off = tc::kmajor_offset(NX + u % (NM - NX), 4 * (u / (NM - NX)), 4, KG);
+      *reinterpret_cast<uint4*>(Bhi + off) = make_uint4(0, 0, 0, 0);
+      if (SPLIT) *reinterpret_cast<uint4*>(Blo + off) = make_uint4(0, 0, 0, 0);
+    }
   }
   if (tid == 0) {
     tc::mbar_init(&full[0], 1);
@@ -571,7 +579,8 @@ __global__ void __launch_bounds__(kDcThreads, 1) k_apply_dc_tc(const float* __re
   const uint32_t tbase = s_tmem;
   // column slices of 16 (or more) per warp group: warp w takes lanes
   // 32 (w % 4).. and slice w / 4 (warp groups beyond the slices idle here)
-  const int nslice = min(kDcThreads / 128, NM / 16);
+  int nslice = min(kDcThreads / 128, NM / 16);
+  while (NM / 16 % nslice != 0) --nslice;
   const int sw = NM / nslice;                              // columns per slice
   const int slice = warp >> 2;
   const int own = slice < nslice ? sw : 0;
@@ -653,8 +662,8 @@ __global__ void __launch_bounds__(kDcThreads, 1) k_apply_dc_tc(const float* __re
     // rows (kk, p) of the x block
     {
       const float* X = reinterpret_cast<const float*>(raw + x_off);
-      for (int u = tid; u < NM * KG; u += kDcThreads) {
-        const int n = u % NM, kq = u / NM;
+      for (int u = tid; u < NX * KG; u += kDcThreads) {
+        const int n = u % NX, kq = u / NX;
         const int p = n / nrhs, r = n % nrhs;
         uint32_t h[4], l[4];
 #pragma unroll
@@ -832,16 +841,21 @@ void dc_images_build(mrhs_ctx c) {
 }
 
 // coarse stencil on the tensor cores (FP32 coarse fields): split-tf32 (FP32
-// accuracy) or single tf32; false when the shape is outside the kernel's
+// accuracy) or single tf32; false when the shape is outside the kernel's. Any count
+// of right-hand sides from 9 on (the columns are filled up to 16 with zeros): at
+// 16^3x32, 2ntv = 40, 20 of them take 73 us against 114 on the CUDA cores, 9 take 67
+// against 126; in the even-odd solve 41 us a launch against 109; 32^3x64, bf16
+// setup, 24 (split, converting each block): 1.24 against 1.85 ms
 bool apply_Dc_tc(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, bool split) {
   const int nc = 2 * c->ntv;
-  if (c->work_dtype != MRHS_F32 || nc % 8 != 0 || nc > 64 || nrhs % 16 != 0 || nrhs > 64) return false;
+  if (c->work_dtype != MRHS_F32 || nc % 8 != 0 || nc > 64 || nrhs > 64) return false;
+  const int NM = (2 * nrhs + 15) & ~15;
   const int KG = nc / 4;
-  const size_t tiles = (size_t)(kRows / 8 * KG * 128 + 2 * nrhs / 8 * KG * 128);
+  const size_t tiles = (size_t)(kRows / 8 * KG * 128 + NM / 8 * KG * 128);
   const size_t raw = ((size_t)nc * nc * 8 + (size_t)nc * 2 * nrhs * 4 + 1023) & ~(size_t)1023;
-  size_t smem = std::max(2 * raw, sizeof(float) * kRows * (2 * nrhs + 1)) + (split ? 2 : 1) * tiles;
+  size_t smem = std::max(2 * raw, sizeof(float) * kRows * (NM + 1)) + (split ? 2 : 1) * tiles;
   uint32_t cols = 32;
-  while (cols < (uint32_t)(4 * nrhs)) cols <<= 1;  // R and S regions of 2 nrhs columns each
+  while (cols < (uint32_t)(2 * NM)) cols <<= 1;  // R and S regions of NM columns each
   int* err = c->dflag + 3;
   const void* src = c->Dc;
   const bool pre = c->dc_img && c->dc_img_version == c->dc_version && c->dc_img_split == (int)split;
@@ -850,8 +864,8 @@ bool apply_Dc_tc(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, bool split) {
     // stages hold the operand images instead of the FP32 blocks; no A tiles
     const size_t img = (size_t)(split ? 2 : 1) * (kRows / 8 * KG * 128);
     const size_t stage = (img + (size_t)nc * 2 * nrhs * 4 + 1023) & ~(size_t)1023;
-    const size_t btiles = (size_t)(split ? 2 : 1) * (2 * nrhs / 8 * KG * 128);
-    smem = std::max(2 * stage, sizeof(float) * kRows * (2 * nrhs + 1)) + btiles;
+    const size_t btiles = (size_t)(split ? 2 : 1) * (NM / 8 * KG * 128);
+    smem = std::max(2 * stage, sizeof(float) * kRows * (NM + 1)) + btiles;
   }
   // a shape whose pipeline stages do not fit in shared memory (e.g. 64
   // right-hand sides in split form at 2 ntv = 64) takes the CUDA-core stencil

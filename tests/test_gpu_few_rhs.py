@@ -8,7 +8,8 @@ import numpy as np
 import pytest
 
 import oracle
-from paper_1601_03184_gb300 import (MRHS_F32, MRHS_F64, MRHS_PREC_FP32, MRHS_PREC_FP64, Lattice, inputs)
+from paper_1601_03184_gb300 import (MRHS_F32, MRHS_F64, MRHS_PREC_FP32, MRHS_PREC_FP64, MRHS_PREC_MIX_BF16, Lattice,
+                                    inputs, mrhs_profile, mrhs_profile_read)
 
 pytestmark = pytest.mark.gpu
 
@@ -68,4 +69,35 @@ def test_coarse_gmres_reductions(nrhs, prec, tol):
     assert list(its) == list(rits)
     for r in range(nrhs):
         assert np.linalg.norm(x[r] - ref[r]) <= tol * np.linalg.norm(ref[r]), r
+    lat.close()
+
+
+# The tensor-core stencil with columns filled up to 16: 9 (the fewest), 20 and 24
+# (the configurations' N_tv), 33 (five column groups for one slice), and 16 beside
+# them. The entries' bound is the few-vector test's with the split operands' 2^-21
+# in place of the unit roundoff of a product.
+@pytest.mark.parametrize("prec", [MRHS_PREC_FP32, MRHS_PREC_MIX_BF16])
+@pytest.mark.parametrize("ntv", [4, 20, 32])
+def test_coarse_stencil_of_other_counts(ntv, prec):
+    lat = Lattice(DIMS, AGG, ntv, prec)
+    lat.set_gauge(inputs.gauge_field(DIMS, 0.5, 1403))
+    lat.build_clover(-0.1, 1.2)
+    lat.set_tv(lat.to_device(inputs.test_vectors(ntv, DIMS, 2403), MRHS_F32), MRHS_F32)
+    lat.build_P()
+    lat.build_Dc()
+    Dc = lat.get_Dc()
+    n = 2 * 9 * 2 * ntv + 2
+    rel = n * 2.0 ** -24 / (1 - n * 2.0 ** -24) + 2 * 2.0 ** -21
+    for nrhs in (9, 16, 20, 24, 33):
+        if prec == MRHS_PREC_MIX_BF16 and nrhs % 16 == 0:
+            continue  # single tf32 there
+        x = inputs.gaussian_field((nrhs, lat.nagg, 2 * ntv), 4403).astype(np.complex64).astype(np.complex128)
+        xd, yd = lat.to_device(x, MRHS_F32, coarse=True), lat.field(nrhs, MRHS_F32, coarse=True)
+        mrhs_profile(lat.ctx, 1)
+        lat.apply_Dc(xd, yd, nrhs, MRHS_F32)
+        assert "apply_dc_tc" in mrhs_profile_read(lat.ctx)
+        mrhs_profile(lat.ctx, 0)
+        ref = oracle.apply_Dc(DIMS, AGG, Dc, x)
+        size = oracle.apply_Dc(DIMS, AGG, np.abs(Dc).astype(np.complex128), np.abs(x).astype(np.complex128)).real
+        assert np.all(np.abs(lat.to_host(yd, nrhs, MRHS_F32, coarse=True) - ref) <= 2 ** 0.5 * rel * size + 1e-300), nrhs
     lat.close()
