@@ -77,7 +77,7 @@ def test_coarse_gmres_reductions(nrhs, prec, tol):
 # them. The entries' bound is the few-vector test's with the split operands' 2^-21
 # in place of the unit roundoff of a product.
 @pytest.mark.parametrize("prec", [MRHS_PREC_FP32, MRHS_PREC_MIX_BF16])
-@pytest.mark.parametrize("ntv", [4, 20, 32])
+@pytest.mark.parametrize("ntv", [8, 20, 32])
 def test_coarse_stencil_of_other_counts(ntv, prec):
     lat = Lattice(DIMS, AGG, ntv, prec)
     lat.set_gauge(inputs.gauge_field(DIMS, 0.5, 1403))
