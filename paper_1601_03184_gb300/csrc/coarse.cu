@@ -662,25 +662,48 @@ __global__ void k_prolong6(const SP* __restrict__ P, const SC* __restrict__ uc, 
   for (int cc = 0; cc < 6; ++cc) st<SU, R>(u, s * 12 + 6 * h + cc, N, r, acc[cc]);
 }
 
-// The same for FP32 fields with N % 4 == 0 and Nt % 4 == 0: per (aggregate, chirality)
-// the product of the 6 Va x Nt rows of P with the Nt x N coarse block, which is staged
-// in shared memory; a thread holds four fine rows and four right-hand sides, and reads
+// W consecutive values of a row in FP32, W 4, 2 or 1
+template <int W, class S>
+__device__ __forceinline__ void ld_some(const S* p, float* v) {
+  if constexpr (W == 4) {
+    ld_four(p, v);
+  } else if constexpr (W == 2 && sizeof(S) == 2) {
+    const uint32_t t = __ldg(reinterpret_cast<const uint32_t*>(p));
+    S h[2];
+    *reinterpret_cast<uint32_t*>(h) = t;
+    v[0] = to_r(h[0]), v[1] = to_r(h[1]);
+  } else if constexpr (W == 2 && sizeof(S) == 4) {
+    const float2 t = __ldg(reinterpret_cast<const float2*>(p));
+    v[0] = t.x, v[1] = t.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < W; ++i) v[i] = (float)to_r(p[i]);
+  }
+}
+
+// The same for FP32 fields with N % 4 == 0: per (aggregate, chirality) the product of
+// the 6 Va x Nt rows of P with the Nt x N coarse block, which is staged in shared
+// memory, QC groups of four columns to a CTA; a thread holds four fine rows and four right-hand sides, and reads
 // four columns j of its rows of P at once: sixteen 16-byte reads feed 256 FMAs, where one
 // site's six rows and a single column per step took fourteen reads for 96. The sums
 // run over j in order, as in the other forms. Per call, before and after: 512
 // aggregates, 32 x 32, FP32: 514 -> 326 us; 8192, 24 x 24, bf16 P: 4822 -> 3112 us.
+// W: columns of P in one load, the largest of 4, 2 and 1 that divides Nt (a row
+// starts on a multiple of W only then); W = 1 still takes four columns a step. 16^4,
+// FP32, before (a thread with one site's six rows) and after: 13 x 8 63 -> 54 us,
+// 13 x 24 104 -> 90, 6 x 8 29 -> 28; bf16 P: 10 x 8 36 -> 32, 13 x 8 45 -> 48.
 constexpr int kProRows = 4;
-template <class SP>
+template <class SP, int W>
 __global__ void __launch_bounds__(256) k_prolong_tile(const SP* __restrict__ P, const float* __restrict__ uc,
-                                                      float* __restrict__ u, int Nt, int N, int Va) {
+                                                      float* __restrict__ u, int Nt, int N, int Va, int QC) {
   extern __shared__ double smem_d[];
-  float4* w = reinterpret_cast<float4*>(smem_d);  // [Nt][2][N / 4]
-  const int A = blockIdx.x >> 1, h = blockIdx.x & 1, Q = N / 4;
-  const float4* src = reinterpret_cast<const float4*>(uc + ((size_t)A * 2 + h) * Nt * 2 * N);
-  for (int i = threadIdx.x; i < Nt * 2 * Q; i += 256) w[i] = __ldg(src + i);
+  float4* w = reinterpret_cast<float4*>(smem_d);  // [Nt][2][Q]
+  const int A = blockIdx.x >> 1, h = blockIdx.x & 1, q0 = blockIdx.z * QC, Q = min(QC, N / 4 - q0);
+  const float4* src = reinterpret_cast<const float4*>(uc + ((size_t)A * 2 + h) * Nt * 2 * N) + q0;
+  for (int i = threadIdx.x; i < Nt * 2 * Q; i += blockDim.x) w[i] = __ldg(src + i / Q * (N / 4) + i % Q);
   __syncthreads();
   const int nrow = 6 * Va, ng = (nrow + kProRows - 1) / kProRows;
-  for (int t = blockIdx.y * 256 + threadIdx.x; t < ng * Q; t += gridDim.y * 256) {
+  for (int t = blockIdx.y * blockDim.x + threadIdx.x; t < ng * Q; t += gridDim.y * blockDim.x) {
     const int q = t % Q, l0 = t / Q * kProRows;
     size_t row[kProRows];
 #pragma unroll
@@ -693,15 +716,18 @@ __global__ void __launch_bounds__(256) k_prolong_tile(const SP* __restrict__ P, 
     for (int a = 0; a < kProRows; ++a)
 #pragma unroll
       for (int e = 0; e < 4; ++e) are[a][e] = aim[a][e] = 0.f;
-    for (int j = 0; j < Nt; j += 4) {
-      float pr[kProRows][4], pi[kProRows][4];
+    auto columns = [&](auto count, int j) {  // columns j .. j + count - 1
+      constexpr int C = decltype(count)::value;
+      float pr[kProRows][C], pi[kProRows][C];
 #pragma unroll
-      for (int a = 0; a < kProRows; ++a) {
-        ld_four(P + row[a] * 2 * Nt + j, pr[a]);
-        ld_four(P + row[a] * 2 * Nt + Nt + j, pi[a]);
-      }
+      for (int a = 0; a < kProRows; ++a)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < C; i += W) {
+          ld_some<W>(P + row[a] * 2 * Nt + j + i, pr[a] + i);
+          ld_some<W>(P + row[a] * 2 * Nt + Nt + j + i, pi[a] + i);
+        }
+#pragma unroll
+      for (int i = 0; i < C; ++i) {
         const float4 w0 = w[(j + i) * 2 * Q + q], w1 = w[((j + i) * 2 + 1) * Q + q];
         const float wr[4] = {w0.x, w0.y, w0.z, w0.w}, wi[4] = {w1.x, w1.y, w1.z, w1.w};
 #pragma unroll
@@ -712,12 +738,17 @@ __global__ void __launch_bounds__(256) k_prolong_tile(const SP* __restrict__ P, 
             aim[a][e] = fmaf(pi[a][i], wr[e], fmaf(pr[a][i], wi[e], aim[a][e]));
           }
       }
-    }
+    };
+    int j = 0;
+    if (W != 2)
+      for (; j + 4 <= Nt; j += 4) columns(std::integral_constant<int, 4>{}, j);
+    if (W != 4)
+      for (; j < Nt; j += W) columns(std::integral_constant<int, W>{}, j);
 #pragma unroll
     for (int a = 0; a < kProRows; ++a)
       if (l0 + a < nrow) {
-        *reinterpret_cast<float4*>(u + fidx(row[a], 0, N, 4 * q)) = make_float4(are[a][0], are[a][1], are[a][2], are[a][3]);
-        *reinterpret_cast<float4*>(u + fidx(row[a], 1, N, 4 * q)) = make_float4(aim[a][0], aim[a][1], aim[a][2], aim[a][3]);
+        *reinterpret_cast<float4*>(u + fidx(row[a], 0, N, 4 * (q0 + q))) = make_float4(are[a][0], are[a][1], are[a][2], are[a][3]);
+        *reinterpret_cast<float4*>(u + fidx(row[a], 1, N, 4 * (q0 + q))) = make_float4(aim[a][0], aim[a][1], aim[a][2], aim[a][3]);
       }
   }
 }
@@ -1074,11 +1105,21 @@ void prolong_typed(mrhs_ctx c, const void* uc, int dc, void* u, int du, int N) {
   size_t work = (size_t)c->g.V * 2 * N;
   Prof pr(c, "prolong");
   const bool aligned = ((uintptr_t)uc & 15) == 0 && ((uintptr_t)u & 15) == 0;
-  const size_t smem = sizeof(float) * 2 * (size_t)c->ntv * N;
-  if (dc == MRHS_F32 && du == MRHS_F32 && c->ntv % 4 == 0 && N % 4 == 0 && aligned && smem <= 48 * 1024) {
-    // (two rounds of a CTA's threads over its rows: the coarse block staged serves them)
-    const dim3 grid(2 * c->g.nagg, std::max(1, 6 * c->g.Va / kProRows * (N / 4) / 512));
-    MRHS_DISPATCH(c->tv_dtype, SP, (k_prolong_tile<SP><<<grid, 256, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va)));
+  if (dc == MRHS_F32 && du == MRHS_F32 && N % 4 == 0 && aligned) {
+    // the block's columns in pieces of at most 48 KB (Nt <= 64: 24 groups and more), and
+    // two rounds of a CTA's threads over its rows: the coarse block staged serves them
+    const int QC = std::min(N / 4, 48 * 1024 / (32 * c->ntv));
+    const size_t smem = (size_t)32 * c->ntv * QC;
+    const int tiles = (6 * c->g.Va + kProRows - 1) / kProRows * QC, threads = std::min(256, (tiles + 31) / 32 * 32);
+    const dim3 grid(2 * c->g.nagg, std::max(1, tiles / 512), (N / 4 + QC - 1) / QC);
+    MRHS_DISPATCH(c->tv_dtype, SP, {
+      if (c->ntv % 4 == 0)
+        k_prolong_tile<SP, 4><<<grid, threads, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, QC);
+      else if (c->ntv % 2 == 0)
+        k_prolong_tile<SP, 2><<<grid, threads, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, QC);
+      else
+        k_prolong_tile<SP, 1><<<grid, threads, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, QC);
+    });
     MRHS_LAUNCH_CHECK("prolong_tile");
     return;
   }
