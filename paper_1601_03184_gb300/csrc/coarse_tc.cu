@@ -826,7 +826,11 @@ void dc_images_build(mrhs_ctx c) {
     const size_t bytes = nblk * 2 * a_bytes;  // room for either form
     size_t free_b = 0, total_b = 0;
     MRHS_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    if (bytes + ((size_t)1 << 30) > free_b) return;
+    const size_t want = bytes + ((size_t)1 << 30);
+    if (want > free_b) {  // the smoother's tile copies give way: they shrink to what is left
+      if (want > free_b + c->scratch[SC_TILES].bytes) return;
+      release_scratch(c, SC_TILES);
+    }
     c->dc_img = dalloc(c, bytes);
   }
   const size_t n = nblk * (size_t)kRows * KG;

@@ -189,7 +189,8 @@ struct mrhs_ctx_s {
   double* U64 = nullptr;  // [V][4][9] complex
   float* U32 = nullptr;
   float* U20 = nullptr;   // [V][4][20]: FP32 links padded to 80 bytes (float4-aligned records)
-  float* UQ = nullptr;    // [nagg][20][Va][4]: the same, sites innermost (float4 k of link mu at row 5 mu + k)
+  size_t uq_bytes() const { return (size_t)g.V * 80 * sizeof(float); }
+  float* UQ = nullptr;    // (where there was room) [nagg][20][Va][4]: the same, sites innermost (float4 k of link mu at row 5 mu + k)
   double* A64 = nullptr;  // [V][2][36]
   float* A32 = nullptr;
   double* Ainv64 = nullptr;  // [V][2][36] inverse clover term (even-odd smoother), built on first use
@@ -264,6 +265,8 @@ enum Scratch {
 };
 
 void* scratch(mrhs_ctx c, int which, size_t bytes);
+void* scratch_or_null(mrhs_ctx c, int which, size_t bytes);  // nullptr when the memory has run out
+void release_scratch(mrhs_ctx c, int which);
 // refuse (MRHS_ERR_ARG) a caller pointer of the wrong memory type before any
 // launch or copy touches it: require_dev wants device memory of the
 // context's GPU (or managed memory), require_host host memory (pageable,

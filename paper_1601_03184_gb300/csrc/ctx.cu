@@ -5,6 +5,8 @@
 
 #include "common.cuh"
 
+#include <algorithm>
+
 using namespace mrhs;
 
 namespace {
@@ -14,10 +16,52 @@ thread_local std::string g_create_error;
 namespace mrhs {
 std::string& create_error_slot() { return g_create_error; }
 
-void* dalloc(mrhs_ctx c, size_t bytes) {
+// cudaMalloc, or nullptr when the memory has run out
+static void* malloc_or_null(size_t bytes) {
   void* p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  MRHS_CUDA(e);
+  return p;
+}
+
+void release_scratch(mrhs_ctx c, int which) {
+  DevBuf& b = c->scratch[which];
+  if (!b.p) return;
+  MRHS_CUDA(cudaStreamSynchronize(c->stream));
+  MRHS_CUDA(cudaFree(b.p));
+  c->held_bytes -= b.bytes;
+  b.p = nullptr;
+  b.bytes = 0;
+}
+
+// Device memory that is needed: when it has run out, what the context holds only to
+// run faster goes first, the smoother's tile copies and then its links (the smoother
+// works without either), so that the same sizes fit as without them.
+static void* need_malloc(mrhs_ctx c, size_t bytes) {
+  void* p = malloc_or_null(bytes);
+  if (!p && c->scratch[SC_TILES].p) {
+    release_scratch(c, SC_TILES);
+    p = malloc_or_null(bytes);
+  }
+  if (!p && c->UQ) {
+    MRHS_CUDA(cudaStreamSynchronize(c->stream));
+    c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), (void*)c->UQ));
+    MRHS_CUDA(cudaFree(c->UQ));
+    c->held_bytes -= c->uq_bytes();
+    c->UQ = nullptr;
+    p = malloc_or_null(bytes);
+  }
+  if (!p) MRHS_CUDA(cudaErrorMemoryAllocation);
+  return p;
+}
+
+void* dalloc(mrhs_ctx c, size_t bytes) {
   if (bytes == 0) bytes = 16;
-  MRHS_CUDA(cudaMalloc(&p, bytes));
+  void* p = need_malloc(c, bytes);
   c->allocs.push_back(p);
   c->held_bytes += bytes;
   return p;
@@ -26,14 +70,20 @@ void* dalloc(mrhs_ctx c, size_t bytes) {
 void* scratch(mrhs_ctx c, int which, size_t bytes) {
   DevBuf& b = c->scratch[which];
   if (b.bytes < bytes) {
-    if (b.p) {
-      MRHS_CUDA(cudaStreamSynchronize(c->stream));
-      MRHS_CUDA(cudaFree(b.p));
-      c->held_bytes -= b.bytes;
-      b.p = nullptr;
-      b.bytes = 0;
-    }
-    MRHS_CUDA(cudaMalloc(&b.p, bytes));
+    release_scratch(c, which);
+    b.p = need_malloc(c, bytes);
+    b.bytes = bytes;
+    c->held_bytes += bytes;
+  }
+  return b.p;
+}
+
+void* scratch_or_null(mrhs_ctx c, int which, size_t bytes) {
+  DevBuf& b = c->scratch[which];
+  if (b.bytes < bytes) {
+    release_scratch(c, which);
+    b.p = malloc_or_null(bytes);
+    if (!b.p) return nullptr;
     b.bytes = bytes;
     c->held_bytes += bytes;
   }
@@ -754,13 +804,7 @@ int mrhs_trim(mrhs_ctx c) {
   return guarded(c, [&] {
     MRHS_REQUIRE(c, MRHS_ERR_ARG, "null context");
     MRHS_CUDA(cudaStreamSynchronize(c->stream));
-    for (auto& b : c->scratch)
-      if (b.p) {
-        MRHS_CUDA(cudaFree(b.p));
-        c->held_bytes -= b.bytes;
-        b.p = nullptr;
-        b.bytes = 0;
-      }
+    for (int k = 0; k < SC_COUNT; ++k) release_scratch(c, k);
   });
 }
 
@@ -813,8 +857,14 @@ int mrhs_set_gauge(mrhs_ctx c, const double* U) {
       c->U64 = (double*)dalloc(c, n * sizeof(double));
       c->U32 = (float*)dalloc(c, n * sizeof(float));
       c->U20 = (float*)dalloc(c, (size_t)c->g.V * 80 * sizeof(float));
-      // 48^3 x 96: 3.4 GB, for the on-chip smoother of FP32 work fields
-      if (c->work_dtype == MRHS_F32 && c->g.Va > 128 && c->g.Va <= 256) c->UQ = (float*)dalloc(c, (size_t)c->g.V * 80 * sizeof(float));
+    }
+    // 48^3 x 96: 3.4 GB, for the on-chip smoother of FP32 work fields, where there is room
+    if (!c->UQ && c->work_dtype == MRHS_F32 && c->g.Va > 128 && c->g.Va <= 256) {
+      c->UQ = (float*)malloc_or_null(c->uq_bytes());
+      if (c->UQ) {
+        c->allocs.push_back(c->UQ);
+        c->held_bytes += c->uq_bytes();
+      }
     }
     // chunks of sites through the staging buffer bound the extra device memory
     const size_t per_site = 72 * sizeof(double);

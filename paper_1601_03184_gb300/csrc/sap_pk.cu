@@ -1010,9 +1010,9 @@ static SapGeo sap_face_geo(mrhs_ctx c, int T, size_t* smem) {
 
 // Right-hand sides smoothed together on tile copies: all of them when the two
 // copies take at most kTileBytes (or half of what is free), else fewer, so that the
-// largest lattices keep their memory for the setup (48^3 x 96, 32 vectors: 8 at a
-// time, 16 GB). 0: not even four fit, the caller takes the form without copies.
-constexpr size_t kTileBytes = (size_t)20 << 30;
+// largest lattices keep their memory for the setup (48^3 x 96, 32 vectors: 4 at a
+// time, 8 GB). 0: not even four fit, the caller takes the form without copies.
+constexpr size_t kTileBytes = (size_t)10 << 30;
 static int sap_group(mrhs_ctx c, int nrhs) {
   const size_t four = 2 * sizeof(float) * fine_elems(c, 4);
   const size_t held = c->scratch[SC_TILES].bytes;
@@ -1041,7 +1041,8 @@ static bool sap_face(mrhs_ctx c, const void* b, int bdtype, void* x, int nrhs, i
   uint32_t cols = 32;
   while (cols < (uint32_t)(T / 128) * kPWarpCols) cols <<= 1;
   const size_t tiles = sizeof(float) * fine_elems(c, group);
-  float4* xq = (float4*)scratch(c, SC_TILES, 2 * tiles);
+  float4* xq = (float4*)scratch_or_null(c, SC_TILES, 2 * tiles);
+  if (!xq) return false;
   float4* bq = xq + tiles / sizeof(float4);
   MRHS_CUDA(cudaFuncSetAttribute(k_sap_face, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   for (int g0 = 0; g0 < nrhs; g0 += group) {

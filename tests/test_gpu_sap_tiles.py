@@ -7,6 +7,7 @@ the other FP32 smoother forms.
 every site, one direction at a time; (8,8,2,2): the wide directions first."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import paper_1601_03184_gb300 as pkg
@@ -37,6 +38,35 @@ def test_sap_on_tiles(agg, dims, nrhs, n_mr):
     assert "sap_tiles" in pkg.mrhs_profile_read(lat.ctx)
     ref = oracle.sap(dims, agg, U, A, b, x0, 2, n_mr)
     assert rel(lat.to_host(xd, nrhs, MRHS_F32), ref) < 1e-5
+    lat.close()
+
+
+def test_copies_give_way_to_needed_memory():
+    """What the smoother holds only to run faster is released for what a later step
+    cannot do without: with the device filled up after a smoothing, the test vectors
+    (more than is left) are still stored, and the smoother still gives its result
+    (to the bound of the FP32 forms, twice)."""
+    dims, agg, ntv = (16, 16, 16, 16), (4, 4, 4, 4), 16
+    lat = Lattice(dims, agg, ntv, MRHS_PREC_FP32)
+    lat.set_gauge(inputs.gauge_field(dims, 0.4, 1503))
+    lat.build_clover(-0.1, 1.2)
+    b = torch.randn(lat.V * 24 * ntv, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    first, again = torch.zeros_like(b), torch.zeros_like(b)
+    lat.sap(b, first, ntv, MRHS_F32, 2, 2)
+    lat.sync()
+    torch.cuda.empty_cache()
+    held = pkg.mrhs_info(lat.ctx)[5]
+    rest = torch.cuda.mem_get_info()[0] - (48 << 20)
+    fill = torch.empty(rest, dtype=torch.uint8, device="cuda")  # 48 MB left, 100 MB needed
+    try:
+        lat.set_tv(b, MRHS_F32)
+        assert pkg.mrhs_info(lat.ctx)[5] < held  # 200 MB of copies gone, 100 MB of vectors there
+        lat.sap(b, again, ntv, MRHS_F32, 2, 2)
+        lat.sync()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert torch.linalg.vector_norm((first - again).double()) <= 2e-5 * torch.linalg.vector_norm(first.double())
     lat.close()
 
 
