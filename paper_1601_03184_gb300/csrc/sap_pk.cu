@@ -1009,10 +1009,12 @@ static SapGeo sap_face_geo(mrhs_ctx c, int T, size_t* smem) {
 }
 
 // Right-hand sides smoothed together on tile copies: all of them when the two
-// copies take at most kTileBytes (or half of what is free), else fewer, so that the
-// largest lattices keep their memory for the setup (48^3 x 96, 32 vectors: 4 at a
-// time, 8 GB). 0: not even four fit, the caller takes the form without copies.
-constexpr size_t kTileBytes = (size_t)10 << 30;
+// copies take at most kTileBytes (or 3/4 of what is free), else fewer, so that the
+// largest lattices keep their memory for the setup, in multiples of 8: of a row's 128
+// bytes (32 right-hand sides) whole 64-byte pieces come from memory, so copies of four
+// at a time cost as much as of eight (48^3 x 96, 32 vectors, a setup: 545 ms in fours,
+// 236 ms in eights, 16 GB). 0: not even four fit, the caller takes the form without copies.
+constexpr size_t kTileBytes = (size_t)20 << 30;
 static int sap_group(mrhs_ctx c, int nrhs) {
   const size_t four = 2 * sizeof(float) * fine_elems(c, 4);
   const size_t held = c->scratch[SC_TILES].bytes;
@@ -1026,9 +1028,10 @@ static int sap_group(mrhs_ctx c, int nrhs) {
     if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return 4 * (int)(held / four);
     size_t free_b = 0, total_b = 0;
     MRHS_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    room = std::min(room, (free_b + held) / 2);
+    room = std::max(held, std::min(room, (free_b + held) / 4 * 3));
   }
-  return 4 * (int)std::min<size_t>(nrhs / 4, room / four);
+  const int group = 4 * (int)std::min<size_t>(nrhs / 4, room / four);
+  return group < nrhs && group > 8 ? group & ~7 : group;
 }
 
 // the smoother on tile copies; false: they or the kernel do not fit
