@@ -157,6 +157,8 @@ class ClockSampler:
 # the ncu captures summarised in profiles/ (16x16x16x32, N_tv = 32), scaled by
 # the number of sites; None for a kernel whose code changed since its capture
 NCU_TRAFFIC = {
+    "sap_pk": {"bytes": 944.1152e6, "sites": 16 * 16 * 16 * 32, "ntv": 32,
+               "profile": "profiles/k_sap_face_16x16x16x32_ntv32.md"},
     "sap_tm": {"bytes": 903.34e6, "sites": 16 * 16 * 16 * 32, "ntv": 32,
                "profile": "profiles/k_sap_tm_16x16x16x32_ntv32.md"},
 }
