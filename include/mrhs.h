@@ -162,7 +162,12 @@ int mrhs_apply_D_block(mrhs_ctx ctx, const void* x, void* y, int nrhs, int dtype
  * the aggregate coordinates); per colour r = b - D x, then on every domain
  * B of that colour n_mr minimal-residual steps on D_B e = r_B from e = 0
  * (alpha = <q,rho>/<q,q>, q = D_B rho), and x_B += e. b, x: device fields
- * of storage dtype F64 or F32. */
+ * of storage dtype F64 or F32.
+ * FP32 fields on domains of 129 to 256 sites, nrhs a multiple of 4 and at
+ * least two sweeps: works on copies of b and x in a workspace of the context.
+ * A call recorded into a CUDA graph never does: its replays use b, x and the
+ * context's gauge field and clover term only, whatever happens to the
+ * workspace meanwhile. */
 int mrhs_sap(mrhs_ctx ctx, const void* b, void* x, int nrhs, int dtype, int n_sweeps, int n_mr);
 
 /* Domain solves of the SAP smoother (every use: mrhs_sap, the setup phases,

@@ -267,6 +267,7 @@ enum Scratch {
 void* scratch(mrhs_ctx c, int which, size_t bytes);
 void* scratch_or_null(mrhs_ctx c, int which, size_t bytes);  // nullptr when the memory has run out
 void release_scratch(mrhs_ctx c, int which);
+bool capturing(mrhs_ctx c);  // whether the context's stream is being captured into a graph
 // refuse (MRHS_ERR_ARG) a caller pointer of the wrong memory type before any
 // launch or copy touches it: require_dev wants device memory of the
 // context's GPU (or managed memory), require_host host memory (pageable,

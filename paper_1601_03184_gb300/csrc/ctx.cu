@@ -38,6 +38,13 @@ void release_scratch(mrhs_ctx c, int which) {
   b.bytes = 0;
 }
 
+bool capturing(mrhs_ctx c) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
+  if (e != cudaSuccess) cudaGetLastError();  // the legacy stream while another one is captured
+  return e != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+}
+
 // Device memory that is needed: when it has run out, what the context holds only to
 // run faster goes first, the smoother's tile copies and then its links (the smoother
 // works without either), so that the same sizes fit as without them.

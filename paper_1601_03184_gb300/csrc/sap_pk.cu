@@ -1020,12 +1020,6 @@ static int sap_group(mrhs_ctx c, int nrhs) {
   const size_t held = c->scratch[SC_TILES].bytes;
   size_t room = kTileBytes;
   if (held < std::min(room, four * (nrhs / 4))) {
-    // nothing can be allocated while the stream is being captured: the form
-    // without copies, unless an earlier call has left room for four
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
-    if (e != cudaSuccess) cudaGetLastError();
-    if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return 4 * (int)(held / four);
     size_t free_b = 0, total_b = 0;
     MRHS_CUDA(cudaMemGetInfo(&free_b, &total_b));
     room = std::max(held, std::min(room, (free_b + held) / 4 * 3));
@@ -1096,7 +1090,13 @@ void sap_pk(mrhs_ctx c, const void* b, int bdtype, void* x, int nrhs, int n_swee
   }();
   const int cpb = cpb_env > 0 ? std::min(cpb_env, nrhs / kG) : nrhs / kG;
   static const bool switched = std::getenv("MRHS_SAP_PK") || cpb_env > 0;
-  if (!switched && n_sweeps >= 2 && Va > 128 && sap_face(c, b, bdtype, x, nrhs, n_sweeps, n_mr, x0_zero)) return;
+  // A recorded call may be replayed when the copies are long gone (mrhs_trim, a larger
+  // smoothing, an allocation that ran out) or beside a direct call that writes them: while
+  // the stream is captured, the form that touches only the caller's fields and the tables
+  // that live as long as the context.
+  if (!switched && n_sweeps >= 2 && Va > 128 && !capturing(c) &&
+      sap_face(c, b, bdtype, x, nrhs, n_sweeps, n_mr, x0_zero))
+    return;
   for (int sw = 0; sw < n_sweeps; ++sw)
     for (int col = 0; col < 2; ++col) {
       const int* blist = c->blocks_col + (col ? c->ncol[0] : 0);
