@@ -1054,7 +1054,8 @@ void restrict_typed(mrhs_ctx c, const void* v, int dv, void* vc, int dc, int N) 
     const char* e = std::getenv("MRHS_RESTRICT");
     return e && std::string(e) == "tiled";
   }();
-  if (!split_off && dc == MRHS_F32) {
+  // (a caller's field that does not start on 16 bytes takes the forms without wide copies)
+  if (!split_off && dc == MRHS_F32 && ((uintptr_t)v & 15) == 0) {
     const bool vp = Nt % 4 == 0, vv = N % 4 == 0;
     MRHS_DISPATCH(c->tv_dtype, SP, MRHS_DISPATCH(dv, SV, {
       auto kern = N <= 3 && vp ? k_restrict_split<SP, SV, 1, true, false>

@@ -23,6 +23,7 @@
 #include "tc.cuh"
 
 #include <algorithm>
+#include <cstdint>
 #include <cstdlib>
 #include <string>
 
@@ -853,6 +854,7 @@ void dc_images_build(mrhs_ctx c) {
 bool apply_Dc_tc(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, bool split) {
   const int nc = 2 * c->ntv;
   if (c->work_dtype != MRHS_F32 || nc % 8 != 0 || nc > 64 || nrhs > 64) return false;
+  if ((((uintptr_t)pt.x0 | (uintptr_t)pt.xh) & 15) != 0) return false;  // bulk copies start on 16 bytes
   if (nrhs % 16 != 0 && nc < 16) return false;  // K of one MMA: 16^4, 2ntv = 8: 25 to 29 us, 23 on the CUDA cores
   const int NM = (2 * nrhs + 15) & ~15;
   const int KG = nc / 4;

@@ -1028,9 +1028,11 @@ static int sap_group(mrhs_ctx c, int nrhs) {
   return group < nrhs && group > 8 ? group & ~7 : group;
 }
 
-// the smoother on tile copies; false: they or the kernel do not fit
+// the smoother on tile copies; false: they or the kernel do not fit, or b does not
+// start on the 16 bytes that the copies of FP32 fields take at a time
 static bool sap_face(mrhs_ctx c, const void* b, int bdtype, void* x, int nrhs, int n_sweeps, int n_mr, bool x0_zero) {
   const int Va = c->g.Va, T = sap_pk_threads(Va, 1);
+  if (bdtype == MRHS_F32 && ((uintptr_t)b & 15) != 0) return false;
   size_t smem = 0;
   const SapGeo geo = sap_face_geo(c, T, &smem);
   const int group = c->UQ && geo.nF > 0 ? sap_group(c, nrhs) : 0;
