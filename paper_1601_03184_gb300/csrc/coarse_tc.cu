@@ -865,7 +865,11 @@ bool apply_Dc_tc(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, bool split) {
   while (cols < (uint32_t)(2 * NM)) cols <<= 1;  // R and S regions of NM columns each
   int* err = c->dflag + 3;
   const void* src = c->Dc;
-  const bool pre = c->dc_img && c->dc_img_version == c->dc_version && c->dc_img_split == (int)split;
+  bool pre = c->dc_img && c->dc_img_version == c->dc_version && c->dc_img_split == (int)split;
+  // A recorded call is replayed on the D_c of the moment, which the images hold only as
+  // long as every build makes them (not after a change of engine): counts that are not a
+  // multiple of 16 read D_c itself, as they did on the CUDA cores.
+  if (pre && nrhs % 16 != 0 && capturing(c)) pre = false;
   if (pre) {
     src = c->dc_img;
     // stages hold the operand images instead of the FP32 blocks; no A tiles

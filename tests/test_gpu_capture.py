@@ -4,7 +4,7 @@ with its workspaces in between."""
 import pytest
 import torch
 
-from paper_1601_03184_gb300 import MRHS_F32, MRHS_PREC_FP32, Lattice, inputs, mrhs_trim
+from paper_1601_03184_gb300 import MRHS_DC_ALU, MRHS_F32, MRHS_PREC_FP32, Lattice, inputs, mrhs_trim
 
 pytestmark = pytest.mark.gpu
 
@@ -42,4 +42,34 @@ def test_recorded_smoothing_outlives_the_workspace():
             g.replay()
             s.synchronize()
             assert rel(x, direct) <= 2e-5
+        lat.close()
+
+
+def test_recorded_coarse_stencil_follows_the_setup():
+    """20 right-hand sides: after the recording D_c is rebuilt from other test vectors
+    with the CUDA-core engine, which leaves the tensor-core operand images behind; the
+    replay applies the new D_c (each form to FP32 accuracy, 1e-5)."""
+    dims, agg, ntv, n = (8, 8, 8, 8), (4, 4, 4, 4), 8, 20
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        lat = Lattice(dims, agg, ntv, MRHS_PREC_FP32)
+        lat.set_gauge(inputs.gauge_field(dims, 0.4, 1602))
+        lat.build_clover(-0.1, 1.2)
+        for k in range(2):
+            lat.set_tv(lat.to_device(inputs.test_vectors(ntv, dims, 2602 + k), MRHS_F32), MRHS_F32)
+            lat.build_P()
+            lat.build_Dc()
+            if k == 0:
+                x = torch.randn(lat.nagg * 4 * ntv * n, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+                y, direct = torch.zeros_like(x), torch.zeros_like(x)
+                lat.apply_Dc(x, y, n, MRHS_F32)
+                s.synchronize()
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g, stream=s):
+                    lat.apply_Dc(x, y, n, MRHS_F32)
+                lat.set_dc_engine(MRHS_DC_ALU)
+        lat.apply_Dc(x, direct, n, MRHS_F32)
+        g.replay()
+        lat.sync()
+        assert rel(y, direct) <= 2e-5
         lat.close()
