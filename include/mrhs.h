@@ -97,9 +97,9 @@ int mrhs_sync(mrhs_ctx ctx);
  * the library, number of SMs, the CUDA device the context lives on */
 int mrhs_info(mrhs_ctx ctx, long long out[8]);
 
-/* release the context's scratch buffers (work fields, Krylov bases, staging);
- * they are allocated again when a later call needs them. The setup state
- * (test vectors, P, D_c, gauge field, clover) is kept. */
+/* release the context's scratch buffers (work fields, Krylov bases, staging,
+ * the smoother's workspace); they are allocated again when a later call needs
+ * them. The setup state (test vectors, P, D_c, gauge field, clover) is kept. */
 int mrhs_trim(mrhs_ctx ctx);
 
 /* bytes of a device field of nrhs right-hand sides (coarse != 0: coarse
@@ -164,10 +164,14 @@ int mrhs_apply_D_block(mrhs_ctx ctx, const void* x, void* y, int nrhs, int dtype
  * (alpha = <q,rho>/<q,q>, q = D_B rho), and x_B += e. b, x: device fields
  * of storage dtype F64 or F32.
  * FP32 fields on domains of 129 to 256 sites, nrhs a multiple of 4 and at
- * least two sweeps: works on copies of b and x in a workspace of the context.
- * A call recorded into a CUDA graph never does: its replays use b, x and the
- * context's gauge field and clover term only, whatever happens to the
- * workspace meanwhile. */
+ * least two sweeps: works on copies of b and x (and of the links: 320 bytes a
+ * site) in a workspace of at most 20 GB and a quarter of the free memory, taken
+ * for the length of the call and given back in stream order to a memory pool
+ * of the context. The pool keeps it until mrhs_trim or mrhs_destroy, unless a
+ * cudaMalloc of the process needs it: the driver then takes what is idle.
+ * Without room for it the same smoother runs on the fields themselves. So does
+ * a call recorded into a CUDA graph: its replays use b, x and the context's
+ * gauge field and clover term only. The setup phases smooth the same way. */
 int mrhs_sap(mrhs_ctx ctx, const void* b, void* x, int nrhs, int dtype, int n_sweeps, int n_mr);
 
 /* Domain solves of the SAP smoother (every use: mrhs_sap, the setup phases,

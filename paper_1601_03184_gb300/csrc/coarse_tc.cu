@@ -828,9 +828,9 @@ void dc_images_build(mrhs_ctx c) {
     size_t free_b = 0, total_b = 0;
     MRHS_CUDA(cudaMemGetInfo(&free_b, &total_b));
     const size_t want = bytes + ((size_t)1 << 30);
-    if (want > free_b) {  // the smoother's tile copies give way: they shrink to what is left
-      if (want > free_b + c->scratch[SC_TILES].bytes) return;
-      release_scratch(c, SC_TILES);
+    if (want > free_b) {  // the smoother's workspace gives way: it shrinks to what is left
+      if (want > free_b + tiles_held(c)) return;
+      tiles_release(c);
     }
     c->dc_img = dalloc(c, bytes);
   }

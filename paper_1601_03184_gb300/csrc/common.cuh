@@ -189,8 +189,6 @@ struct mrhs_ctx_s {
   double* U64 = nullptr;  // [V][4][9] complex
   float* U32 = nullptr;
   float* U20 = nullptr;   // [V][4][20]: FP32 links padded to 80 bytes (float4-aligned records)
-  size_t uq_bytes() const { return (size_t)g.V * 80 * sizeof(float); }
-  float* UQ = nullptr;    // (where there was room) [nagg][20][Va][4]: the same, sites innermost (float4 k of link mu at row 5 mu + k)
   double* A64 = nullptr;  // [V][2][36]
   float* A32 = nullptr;
   double* Ainv64 = nullptr;  // [V][2][36] inverse clover term (even-odd smoother), built on first use
@@ -226,6 +224,8 @@ struct mrhs_ctx_s {
   // named scratch buffers, grown on demand
   mrhs::DevBuf scratch[20];
 
+  cudaMemPool_t tile_pool = nullptr;  // the on-chip smoother's workspace (ctx.cu)
+
   mrhs::NNState* nn = nullptr;  // learned test-vector generator (nn.cu)
 
   // per-kernel CUDA-event timing (off unless enabled through mrhs_profile)
@@ -260,14 +260,38 @@ enum Scratch {
   SC_EO1,         // even-odd domain solves: rho (even sites) / A^-1 H rho (odd sites)
   SC_EO2,         // q (even) and e (both parities), interleaved as two fields
   SC_COARSE_EO,   // even-odd coarse solve: two operator work fields and bhat
-  SC_TILES,       // tile copies of x and b for the on-chip smoother
   SC_COUNT
 };
 
 void* scratch(mrhs_ctx c, int which, size_t bytes);
-void* scratch_or_null(mrhs_ctx c, int which, size_t bytes);  // nullptr when the memory has run out
 void release_scratch(mrhs_ctx c, int which);
 bool capturing(mrhs_ctx c);  // whether the context's stream is being captured into a graph
+
+// While one of these lives, the thread's calls do not break a capture that another thread
+// or another stream has under way: the pool belongs to this context's stream alone, which
+// is not being captured where the pool is used.
+struct Unrecorded {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  Unrecorded() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~Unrecorded() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// The on-chip smoother's workspace: taken from a pool of the context for one call and
+// given back in stream order, without a synchronisation. Between calls the pool keeps its
+// memory, but as idle pool memory: a cudaMalloc of this process that would run out (of
+// another context, of the caller's own allocator) gets it from the driver. (With what a
+// pool gives back at every synchronisation, or plain allocations, a smoothing of 24 vectors
+// of 32^3 x 64 took 129 ms against 107.)
+struct TileSpace {
+  mrhs_ctx c;
+  void* p = nullptr;  // nullptr when the memory has run out
+  TileSpace(mrhs_ctx ctx, size_t bytes);
+  ~TileSpace();
+  TileSpace(const TileSpace&) = delete;
+  TileSpace& operator=(const TileSpace&) = delete;
+};
+size_t tiles_held(mrhs_ctx c);   // bytes of the pool
+void tiles_release(mrhs_ctx c);  // give them back now (synchronises)
 // refuse (MRHS_ERR_ARG) a caller pointer of the wrong memory type before any
 // launch or copy touches it: require_dev wants device memory of the
 // context's GPU (or managed memory), require_host host memory (pageable,

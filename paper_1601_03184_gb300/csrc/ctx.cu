@@ -6,6 +6,7 @@
 #include "common.cuh"
 
 #include <algorithm>
+#include <cstdint>
 
 using namespace mrhs;
 
@@ -45,21 +46,56 @@ bool capturing(mrhs_ctx c) {
   return e != cudaSuccess || cap != cudaStreamCaptureStatusNone;
 }
 
-// Device memory that is needed: when it has run out, what the context holds only to
-// run faster goes first, the smoother's tile copies and then its links (the smoother
-// works without either), so that the same sizes fit as without them.
+size_t tiles_held(mrhs_ctx c) {
+  if (!c->tile_pool) return 0;
+  const Unrecorded u;
+  uint64_t v = 0;
+  MRHS_CUDA(cudaMemPoolGetAttribute(c->tile_pool, cudaMemPoolAttrReservedMemCurrent, &v));
+  return (size_t)v;
+}
+
+void tiles_release(mrhs_ctx c) {
+  if (!c->tile_pool) return;
+  const Unrecorded u;
+  MRHS_CUDA(cudaStreamSynchronize(c->stream));
+  MRHS_CUDA(cudaMemPoolTrimTo(c->tile_pool, 0));
+}
+
+TileSpace::TileSpace(mrhs_ctx ctx, size_t bytes) : c(ctx) {
+  const Unrecorded u;
+  if (!c->tile_pool) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = c->device;
+    MRHS_CUDA(cudaMemPoolCreate(&c->tile_pool, &props));
+    uint64_t keep = ~0ull;  // idle memory stays mapped: mapping 10 GB takes 20 ms
+    MRHS_CUDA(cudaMemPoolSetAttribute(c->tile_pool, cudaMemPoolAttrReleaseThreshold, &keep));
+  }
+  // a larger workspace takes the place of the one before it
+  if (bytes > tiles_held(c)) MRHS_CUDA(cudaMemPoolTrimTo(c->tile_pool, 0));
+  for (int attempt = 0;; ++attempt) {
+    const cudaError_t e = cudaMallocFromPoolAsync(&p, bytes, c->tile_pool, c->stream);
+    if (e == cudaSuccess) return;
+    p = nullptr;
+    if (e != cudaErrorMemoryAllocation) MRHS_CUDA(e);
+    cudaGetLastError();
+    if (attempt > 0 || tiles_held(c) == 0) return;
+    tiles_release(c);
+  }
+}
+TileSpace::~TileSpace() {
+  const Unrecorded u;
+  if (p) cudaFreeAsync(p, c->stream);
+}
+
+// Device memory that is needed: when it has run out, what the smoother's pool holds goes
+// first (the smoother works without it), so that the same sizes fit as without it.
 static void* need_malloc(mrhs_ctx c, size_t bytes) {
   void* p = malloc_or_null(bytes);
-  if (!p && c->scratch[SC_TILES].p) {
-    release_scratch(c, SC_TILES);
-    p = malloc_or_null(bytes);
-  }
-  if (!p && c->UQ) {
-    MRHS_CUDA(cudaStreamSynchronize(c->stream));
-    c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), (void*)c->UQ));
-    MRHS_CUDA(cudaFree(c->UQ));
-    c->held_bytes -= c->uq_bytes();
-    c->UQ = nullptr;
+  if (!p && tiles_held(c) > 0) {
+    tiles_release(c);
     p = malloc_or_null(bytes);
   }
   if (!p) MRHS_CUDA(cudaErrorMemoryAllocation);
@@ -79,18 +115,6 @@ void* scratch(mrhs_ctx c, int which, size_t bytes) {
   if (b.bytes < bytes) {
     release_scratch(c, which);
     b.p = need_malloc(c, bytes);
-    b.bytes = bytes;
-    c->held_bytes += bytes;
-  }
-  return b.p;
-}
-
-void* scratch_or_null(mrhs_ctx c, int which, size_t bytes) {
-  DevBuf& b = c->scratch[which];
-  if (b.bytes < bytes) {
-    release_scratch(c, which);
-    b.p = malloc_or_null(bytes);
-    if (!b.p) return nullptr;
     b.bytes = bytes;
     c->held_bytes += bytes;
   }
@@ -208,25 +232,22 @@ __global__ void k_tables_canon(GeomArgs g, const int* nbr, const int* perm, cons
 // factor 1/2 and the antiperiodic sign of a hop across the t boundary belong
 // to the link (the forward hop from x and the backward hop from x+mu cross the
 // boundary together)
-// (UQ, may be null: the same, four floats of a link at a time and the sites of an
-// aggregate innermost: [aggregate][5 mu + k][Va] float4 with k < 5)
 __global__ void k_gauge_in(int s0, int ns, const int* perm, const double* Uc, double* U64, float* U32, float* U20,
-                           float* UQ, int Va, int Lt_last_start) {
+                           int Lt_last_start) {
   size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
   if (t >= (size_t)ns * 80) return;
   size_t s = t / 80, e = t % 80;
   size_t sd = (size_t)perm[s0 + s];
   size_t mu = e / 20, k = e % 20;
-  float u20 = 0.f;
   if (k < 18) {
     double v = Uc[s * 72 + mu * 18 + k];
     U64[sd * 72 + mu * 18 + k] = v;
     U32[sd * 72 + mu * 18 + k] = (float)v;
     const bool flip = mu == 3 && (size_t)(s0 + s) >= (size_t)Lt_last_start;
-    u20 = (float)(flip ? -0.5 * v : 0.5 * v);
+    U20[sd * 80 + e] = (float)(flip ? -0.5 * v : 0.5 * v);
+  } else {
+    U20[sd * 80 + e] = 0.f;
   }
-  U20[sd * 80 + e] = u20;
-  if (UQ) UQ[((sd / Va * 20 + e / 4) * Va + sd % Va) * 4 + e % 4] = u20;
 }
 
 // ------------------------------------------------------------ clover ------
@@ -788,6 +809,7 @@ void mrhs_destroy(mrhs_ctx c) {
   for (void* p : c->allocs) cudaFree(p);
   for (auto& b : c->scratch)
     if (b.p) cudaFree(b.p);
+  if (c->tile_pool) cudaMemPoolDestroy(c->tile_pool);
   for (cudaEvent_t e : c->gm_event)
     if (e) cudaEventDestroy(e);
   if (c->hflag) cudaFreeHost(c->hflag);
@@ -812,6 +834,7 @@ int mrhs_trim(mrhs_ctx c) {
     MRHS_REQUIRE(c, MRHS_ERR_ARG, "null context");
     MRHS_CUDA(cudaStreamSynchronize(c->stream));
     for (int k = 0; k < SC_COUNT; ++k) release_scratch(c, k);
+    tiles_release(c);
   });
 }
 
@@ -823,7 +846,7 @@ int mrhs_info(mrhs_ctx c, long long out[8]) {
     out[2] = c->g.Va;
     out[3] = c->ntv;
     out[4] = c->prec;
-    out[5] = (long long)c->held_bytes;
+    out[5] = (long long)(c->held_bytes + tiles_held(c));
     out[6] = c->num_sms;
     out[7] = c->device;
   });
@@ -865,14 +888,6 @@ int mrhs_set_gauge(mrhs_ctx c, const double* U) {
       c->U32 = (float*)dalloc(c, n * sizeof(float));
       c->U20 = (float*)dalloc(c, (size_t)c->g.V * 80 * sizeof(float));
     }
-    // 48^3 x 96: 3.4 GB, for the on-chip smoother of FP32 work fields, where there is room
-    if (!c->UQ && c->work_dtype == MRHS_F32 && c->g.Va > 128 && c->g.Va <= 256) {
-      c->UQ = (float*)malloc_or_null(c->uq_bytes());
-      if (c->UQ) {
-        c->allocs.push_back(c->UQ);
-        c->held_bytes += c->uq_bytes();
-      }
-    }
     // chunks of sites through the staging buffer bound the extra device memory
     const size_t per_site = 72 * sizeof(double);
     const size_t chunk = std::max<size_t>(1, std::min<size_t>(c->g.V, (size_t(1) << 30) / per_site));
@@ -882,7 +897,7 @@ int mrhs_set_gauge(mrhs_ctx c, const double* U) {
       MRHS_CUDA(cudaMemcpyAsync(st, U + s0 * 72, ns * per_site, cudaMemcpyHostToDevice, c->stream));
       const int lt_last = c->g.L[0] * c->g.L[1] * c->g.L[2] * (c->g.L[3] - 1);  // first canonical site with t = Lt-1
       k_gauge_in<<<grid_for((size_t)ns * 80, 256), 256, 0, c->stream>>>((int)s0, ns, c->perm, st, c->U64, c->U32, c->U20,
-                                                                       c->UQ, c->g.Va, lt_last);
+                                                                       lt_last);
       MRHS_LAUNCH_CHECK("gauge_in");
     }
     MRHS_CUDA(cudaStreamSynchronize(c->stream));

@@ -675,8 +675,8 @@ void nn_infer(mrhs_ctx c, const float* in, float* out, int N) {
   const size_t per_rhs = sizeof(float) * (size_t)c->g.V * (2 * (size_t)hid * 6 + 2 * 24);
   size_t free_b = 0, total_b = 0;
   MRHS_CUDA(cudaMemGetInfo(&free_b, &total_b));
-  size_t avail = free_b;
-  for (int k : {SC_FINE1, SC_FINE2, SC_FINE3, SC_TILES}) avail += c->scratch[k].bytes;  // reusable, or given back
+  size_t avail = free_b + tiles_held(c);
+  for (int k : {SC_FINE1, SC_FINE2, SC_FINE3}) avail += c->scratch[k].bytes;  // reusable, or given back
   int chunk = 8;
   while (chunk > 1 && (size_t)chunk * per_rhs > avail / 2) --chunk;
   nn_infer_chunked(c, in, out, N, chunk);

@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(256 * PP, 3 - PP) k_sap_pk(const SB* __restric
 //     pass per direction over the sites at either face: a lane at the forward face
 //     takes U h, one at the backward face U^dag h', with the signs and the
 //     conjugate-transposed link selected per lane;
-//   - the links have the sites innermost (UQ), so that a warp's 16-byte loads fall
+//   - the links have the sites innermost (k_links), so that a warp's 16-byte loads fall
 //     into 4 lines each, not 32.
 // What bounds it now: the packed FMAs (9,000 cycles of the 11,000 to 13,000 that two
 // CTAs take for an application of D_B side by side) and, in the residual, the
@@ -892,6 +892,25 @@ __global__ void __launch_bounds__(256, 2) k_sap_face(const float4* __restrict__ 
   if (warp == 0) tc::tmem_dealloc(s_tmem, tm_cols);
 }
 
+// the links with the sites of a domain innermost: float4 k of link mu at row 5 mu + k of
+// [domain][20][Va]. Made anew by every call (a read and a write of 320 bytes a site, 42 MB
+// each at 16^3 x 32) rather than held by the context beside U20. CTA (domain, kLinkSites
+// of its sites), through shared memory (rows of 21 float4: reads of a column fall into
+// different banks), so that both sides are runs of 1 KB and more.
+constexpr int kLinkSites = 64;
+__global__ void __launch_bounds__(256) k_links(const float4* __restrict__ U20, float4* __restrict__ UQ, int Va) {
+  __shared__ float4 sm[kLinkSites * 21];
+  const int l0 = blockIdx.y * kLinkSites, n = min(kLinkSites, Va - l0);
+  const float4* src = U20 + ((size_t)blockIdx.x * Va + l0) * 20;
+  float4* dst = UQ + (size_t)blockIdx.x * 20 * Va + l0;
+  for (int i = threadIdx.x; i < 20 * n; i += 256) sm[i / 20 * 21 + i % 20] = __ldg(src + i);
+  __syncthreads();
+  for (int i = threadIdx.x; i < 20 * kLinkSites; i += 256) {
+    const int l = i % kLinkSites, row = i / kLinkSites;
+    if (l < n) dst[row * Va + l] = sm[l * 21 + row];
+  }
+}
+
 // four consecutive right-hand sides of a row, FP32
 __device__ __forceinline__ float4 ld_four(const float* p) { return *reinterpret_cast<const float4*>(p); }
 template <class S>
@@ -1008,23 +1027,25 @@ static SapGeo sap_face_geo(mrhs_ctx c, int T, size_t* smem) {
   return g;
 }
 
-// Right-hand sides smoothed together on tile copies: all of them when the two
-// copies take at most kTileBytes (or 3/4 of what is free), else fewer, so that the
-// largest lattices keep their memory for the setup, in multiples of 8: of a row's 128
-// bytes (32 right-hand sides) whole 64-byte pieces come from memory, so copies of four
+// Right-hand sides smoothed together on tile copies: all of them when the workspace (the
+// links and two copies) takes at most kTileBytes (or a quarter of what is free), else fewer, so
+// that the largest lattices keep their memory for the setup, in multiples of 8: of a row's
+// 128 bytes (32 right-hand sides) whole 64-byte pieces come from memory, so copies of four
 // at a time cost as much as of eight (48^3 x 96, 32 vectors, a setup: 545 ms in fours,
 // 236 ms in eights, 16 GB). 0: not even four fit, the caller takes the form without copies.
 constexpr size_t kTileBytes = (size_t)20 << 30;
-static int sap_group(mrhs_ctx c, int nrhs) {
+static int sap_group(mrhs_ctx c, int nrhs, size_t links) {
   const size_t four = 2 * sizeof(float) * fine_elems(c, 4);
-  const size_t held = c->scratch[SC_TILES].bytes;
+  const size_t held = tiles_held(c);
   size_t room = kTileBytes;
-  if (held < std::min(room, four * (nrhs / 4))) {
+  if (held < std::min(room, links + four * (nrhs / 4))) {
+    const Unrecorded u;
     size_t free_b = 0, total_b = 0;
     MRHS_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    room = std::max(held, std::min(room, (free_b + held) / 4 * 3));
+    room = std::max(held, std::min(room, (free_b + held) / 4));
   }
-  const int group = 4 * (int)std::min<size_t>(nrhs / 4, room / four);
+  if (room < links + four) return 0;
+  const int group = 4 * (int)std::min<size_t>(nrhs / 4, (room - links) / four);
   return group < nrhs && group > 8 ? group & ~7 : group;
 }
 
@@ -1032,16 +1053,20 @@ static int sap_group(mrhs_ctx c, int nrhs) {
 // start on the 16 bytes that the copies of FP32 fields take at a time
 static bool sap_face(mrhs_ctx c, const void* b, int bdtype, void* x, int nrhs, int n_sweeps, int n_mr, bool x0_zero) {
   const int Va = c->g.Va, T = sap_pk_threads(Va, 1);
+  if (c->work_dtype != MRHS_F32) return false;
   if (bdtype == MRHS_F32 && ((uintptr_t)b & 15) != 0) return false;
   size_t smem = 0;
   const SapGeo geo = sap_face_geo(c, T, &smem);
-  const int group = c->UQ && geo.nF > 0 ? sap_group(c, nrhs) : 0;
+  const size_t links = sizeof(float) * 80 * c->g.V;
+  const int group = geo.nF > 0 ? sap_group(c, nrhs, links) : 0;
   if (group == 0) return false;
   uint32_t cols = 32;
   while (cols < (uint32_t)(T / 128) * kPWarpCols) cols <<= 1;
   const size_t tiles = sizeof(float) * fine_elems(c, group);
-  float4* xq = (float4*)scratch_or_null(c, SC_TILES, 2 * tiles);
-  if (!xq) return false;
+  const TileSpace ws(c, links + 2 * tiles);
+  if (!ws.p) return false;
+  float4* uq = (float4*)ws.p;
+  float4* xq = uq + links / sizeof(float4);
   float4* bq = xq + tiles / sizeof(float4);
   MRHS_CUDA(cudaFuncSetAttribute(k_sap_face, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   for (int g0 = 0; g0 < nrhs; g0 += group) {
@@ -1051,6 +1076,8 @@ static bool sap_face(mrhs_ctx c, const void* b, int bdtype, void* x, int nrhs, i
     const dim3 grid(c->g.nagg, 12, (Va + ns - 1) / ns);
     {
       Prof pr(c, "sap_tiles");
+      if (g0 == 0)
+        k_links<<<dim3(c->g.nagg, (Va + kLinkSites - 1) / kLinkSites), 256, 0, c->stream>>>((const float4*)c->U20, uq, Va);
       MRHS_DISPATCH(bdtype, SB, (k_tiles<const SB, false><<<grid, 256, smem_t, c->stream>>>((const SB*)b, bq, nrhs, g0, G, Va, ns)));
       if (x0_zero) MRHS_CUDA(cudaMemsetAsync(xq, 0, sizeof(float) * fine_elems(c, G), c->stream));
       else k_tiles<const float, false><<<grid, 256, smem_t, c->stream>>>((const float*)x, xq, nrhs, g0, G, Va, ns);
@@ -1060,9 +1087,8 @@ static bool sap_face(mrhs_ctx c, const void* b, int bdtype, void* x, int nrhs, i
       for (int col = 0; col < 2; ++col) {
         const int* blist = c->blocks_col + (col ? c->ncol[0] : 0);
         Prof pr(c, "sap_pk");
-        k_sap_face<<<c->ncol[col] * nch, T, smem, c->stream>>>(bq, xq, (const float4*)c->UQ, c->A32, c->aggnbr, nch, Va,
-                                                               blist, n_mr, cols, x0_zero && sw == 0 && col == 0,
-                                                                   geo);
+        k_sap_face<<<c->ncol[col] * nch, T, smem, c->stream>>>(bq, xq, uq, c->A32, c->aggnbr, nch, Va, blist, n_mr, cols,
+                                                               x0_zero && sw == 0 && col == 0, geo);
         MRHS_LAUNCH_CHECK("sap_face");
       }
     Prof pr(c, "sap_tiles");
@@ -1092,25 +1118,26 @@ void sap_pk(mrhs_ctx c, const void* b, int bdtype, void* x, int nrhs, int n_swee
   }();
   const int cpb = cpb_env > 0 ? std::min(cpb_env, nrhs / kG) : nrhs / kG;
   static const bool switched = std::getenv("MRHS_SAP_PK") || cpb_env > 0;
-  // A recorded call may be replayed when the copies are long gone (mrhs_trim, a larger
-  // smoothing, an allocation that ran out) or beside a direct call that writes them: while
-  // the stream is captured, the form that touches only the caller's fields and the tables
-  // that live as long as the context.
-  if (!switched && n_sweeps >= 2 && Va > 128 && !capturing(c) &&
-      sap_face(c, b, bdtype, x, nrhs, n_sweeps, n_mr, x0_zero))
-    return;
-  for (int sw = 0; sw < n_sweeps; ++sw)
-    for (int col = 0; col < 2; ++col) {
-      const int* blist = c->blocks_col + (col ? c->ncol[0] : 0);
-      Prof pr(c, "sap_pk");
-      MRHS_DISPATCH(bdtype, SB, {
-        auto kern = f.pp == 1 ? k_sap_pk<SB, 1, true> : f.lg ? k_sap_pk<SB, 2, true> : k_sap_pk<SB, 2, false>;
-        MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  MRHS_DISPATCH(bdtype, SB, {
+    auto kern = f.pp == 1 ? k_sap_pk<SB, 1, true> : f.lg ? k_sap_pk<SB, 2, true> : k_sap_pk<SB, 2, false>;
+    // (in front of both forms: it also loads the kernel, which a first launch inside a
+    // capture must not have to do)
+    MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // The copies live as long as a call, and a recorded call may be replayed at any time,
+    // also beside a direct one: while the stream is captured, the form that touches only
+    // the caller's fields and the tables that live as long as the context.
+    if (!switched && n_sweeps >= 2 && Va > 128 && !capturing(c) &&
+        sap_face(c, b, bdtype, x, nrhs, n_sweeps, n_mr, x0_zero))
+      return;
+    for (int sw = 0; sw < n_sweeps; ++sw)
+      for (int col = 0; col < 2; ++col) {
+        const int* blist = c->blocks_col + (col ? c->ncol[0] : 0);
+        Prof pr(c, "sap_pk");
         kern<<<c->ncol[col] * cpb, T, smem, c->stream>>>((const SB*)b, (float*)x, c->U20, c->A32, c->nbr, nrhs, Va,
                                                          blist, n_mr, cols, cpb, x0_zero && sw == 0 && col == 0);
-      });
-      MRHS_LAUNCH_CHECK("sap_pk");
-    }
+        MRHS_LAUNCH_CHECK("sap_pk");
+      }
+  });
 }
 
 }  // namespace mrhs

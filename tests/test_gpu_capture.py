@@ -73,3 +73,28 @@ def test_recorded_coarse_stencil_follows_the_setup():
         lat.sync()
         assert rel(y, direct) <= 2e-5
         lat.close()
+
+
+def test_direct_smoothing_beside_a_recording():
+    """A smoothing on its own stream while another stream is being captured neither fails
+    nor ends the recording, though it takes its workspace anew each time."""
+    dims, agg, n = (8, 8, 8, 8), (4, 4, 4, 4), 8
+    own, s = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(own):
+        lat = Lattice(dims, agg, 8, MRHS_PREC_FP32)
+        lat.set_gauge(inputs.gauge_field(dims, 0.4, 1603))
+        lat.build_clover(-0.1, 1.2)
+        b = torch.randn(lat.V * 24 * n, device="cuda", generator=torch.Generator("cuda").manual_seed(6))
+        x, y = torch.zeros_like(b), torch.zeros_like(b)
+        lat.sap(b, x, n, MRHS_F32, 2, 3)
+        mrhs_trim(lat.ctx)
+    z = torch.zeros(16, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        z.add_(1)
+        lat.sap(b, y, n, MRHS_F32, 2, 3)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(x, y) and bool((z == 1).all())
+    lat.close()
