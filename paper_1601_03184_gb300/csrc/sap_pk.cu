@@ -1032,20 +1032,22 @@ static SapGeo sap_face_geo(mrhs_ctx c, int T, size_t* smem) {
 // that the largest lattices keep their memory for the setup, in multiples of 8: of a row's
 // 128 bytes (32 right-hand sides) whole 64-byte pieces come from memory, so copies of four
 // at a time cost as much as of eight (48^3 x 96, 32 vectors, a setup: 545 ms in fours,
-// 236 ms in eights, 16 GB). 0: not even four fit, the caller takes the form without copies.
+// 236 ms in eights, 16 GB). A group is at most kTileGroup, so that k_tiles' rows of one
+// site fit in shared memory. 0: not even four fit, the caller takes the form without copies.
 constexpr size_t kTileBytes = (size_t)20 << 30;
+constexpr int kTileGroup = 2048;
 static int sap_group(mrhs_ctx c, int nrhs, size_t links) {
   const size_t four = 2 * sizeof(float) * fine_elems(c, 4);
   const size_t held = tiles_held(c);
   size_t room = kTileBytes;
-  if (held < std::min(room, links + four * (nrhs / 4))) {
+  if (held < std::min(room, links + four * (std::min(nrhs, kTileGroup) / 4))) {
     const Unrecorded u;
     size_t free_b = 0, total_b = 0;
     MRHS_CUDA(cudaMemGetInfo(&free_b, &total_b));
     room = std::max(held, std::min(room, (free_b + held) / 4));
   }
   if (room < links + four) return 0;
-  const int group = 4 * (int)std::min<size_t>(nrhs / 4, (room - links) / four);
+  const int group = std::min(kTileGroup, 4 * (int)std::min<size_t>(nrhs / 4, (room - links) / four));
   return group < nrhs && group > 8 ? group & ~7 : group;
 }
 
