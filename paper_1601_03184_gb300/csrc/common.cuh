@@ -224,7 +224,8 @@ struct mrhs_ctx_s {
   // named scratch buffers, grown on demand
   mrhs::DevBuf scratch[20];
 
-  cudaMemPool_t tile_pool = nullptr;  // the on-chip smoother's workspace (ctx.cu)
+  cudaMemPool_t tile_pool = nullptr;      // the on-chip smoother's workspace (ctx.cu)
+  size_t tile_limit = (size_t)20 << 30;   // and the most that a call takes of it
 
   mrhs::NNState* nn = nullptr;  // learned test-vector generator (nn.cu)
 

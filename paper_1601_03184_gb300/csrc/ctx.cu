@@ -7,6 +7,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <cstdlib>
 
 using namespace mrhs;
 
@@ -758,6 +759,7 @@ int mrhs_create(const int dims[4], const int agg[4], int ntv, int prec, void* st
                     : prec == MRHS_PREC_MIX_BF16 ? MRHS_BF16 : MRHS_F16;
       c->work_dtype = prec == MRHS_PREC_FP64 ? MRHS_F64 : MRHS_F32;
       c->stream = (cudaStream_t)stream;
+      if (const char* e = std::getenv("MRHS_TILE_BYTES")) c->tile_limit = (size_t)std::strtoull(e, nullptr, 10);
       MRHS_CUDA(cudaGetDevice(&c->device));
       MRHS_CUDA(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
       c->nbr = (int*)dalloc(c, sizeof(int) * 8 * (size_t)V);
