@@ -32,16 +32,21 @@ int n_chunks(size_t rows, int N) {
 // 4: FP32, N % 4 == 0, 16-byte loads), Q = N / VEC threads a row, and a warp
 // 32 / Q rows at a time (a row spans warps when Q > 32). Bound by the loads when
 // there are enough rows; at few rows (coarse fields) by the sums across the
-// threads, and there by FP64, which this GPU adds at 2 per clock and SM. So
-// threads of FP32 data with at most kMaxRows rows sum them in FP32, the rows
-// of a warp are joined by FP32 shuffles (a tree: five more roundings) and only
-// the warps' sums are FP64; otherwise (FLUSH) a thread adds its FP32 sums of
-// kFlush rows in FP64 and the threads are joined by a tree in FP64.
+// threads, and there by FP64, which this GPU adds at 2 per clock and SM.
+// Without PAIR a thread adds its (FP32) sums of kFlush rows in FP64 and the threads are
+// joined by a tree in FP64. With PAIR (FP32 data, N <= 32 VEC) a thread sums its rows, at
+// most kMaxRows or with VEC = 1 kFlush, in FP32, and the threads are joined, by shuffles
+// and then across the warps, in pairs of FP32 numbers (two-sums: 48 bits, where the rows'
+// own sums have 24); a pair that leaves the range of FP32 sends the CTA to the same joins
+// in FP64. (Over plain FP32 shuffles, five roundings more, the pairs cost 1 us of a call:
+// a coarse solve of 16^3 x 32 with 32 vectors takes 5.31 ms in place of 5.24.)
 // A chunk is one CTA, or a cluster of eight when the chunks alone would leave
 // most of the GPU idle: the ranks take eighths of the chunk and the first adds
 // their sums in order, so that the partials, and the workspace they need, stay
 // one per chunk.
 constexpr int kKG = 4;          // vectors per group (its sums: up to 40 KB of shared memory)
+constexpr int kKGWide = 2;      // the same for VEC = 4 and more than kWide right-hand sides
+constexpr int kWide = 64;
 constexpr int kFlush = 32;
 constexpr int kMaxRows = 128;
 constexpr int kClusterCtas = 8;
@@ -64,16 +69,23 @@ __device__ __forceinline__ void ld_row(const S* p, typename Real<S>::type v[VEC]
 // rows that one pass of a CTA covers
 __host__ __device__ __forceinline__ int dot_lanes(int Q) { return Q <= 32 ? (kBlock / 32) * (32 / Q) : kBlock / Q; }
 
-template <class S, int VEC, int KG, bool FLUSH>
+// (hi, lo) += (h, l)
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float h, float l) {
+  const float s = __fadd_rn(hi, h), b = __fsub_rn(s, hi);
+  lo = __fadd_rn(__fadd_rn(lo, l), __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(h, b)));
+  hi = s;
+}
+
+template <class S, int VEC, int KG, bool PAIR>
 __global__ void __launch_bounds__(kBlock, 2) k_multi_dot(const S* __restrict__ X, size_t stride, int K,
                                                          const S* __restrict__ Y, size_t rows, int N, int nchunk,
                                                          int ranks, double* __restrict__ part) {
   using R = typename Real<S>::type;
-  // FLUSH: [KG][lanes][N] double2, lanes N <= kBlock; else the warps' sums
-  // [KG][8 warps][N] float2, N <= 128 with VEC = 4 (8 N <= kBlock with VEC = 1,
-  // where wider rows span warps: [KG][lanes][N])
-  __shared__ double2 buf[KG * kBlock * (VEC == 4 ? 2 : 1)];
-  __shared__ double2 res[KG * (VEC == 4 ? 128 : kBlock)];  // [KG][N]
+  // the threads' sums [KG][lanes][N], lanes N <= kBlock; or the warps' pairs
+  // [KG][8 warps][N] float4, KG N <= 64 VEC
+  constexpr int kN = PAIR ? (VEC == 4 ? kBlock : 32 * KG) : KG * kBlock;
+  __shared__ double2 buf[PAIR ? 8 * kN : kN];
+  __shared__ double2 res[kN];  // [KG][N]
   const int k0 = blockIdx.y * KG, ch = blockIdx.x / ranks, rank = blockIdx.x % ranks;
   const int nk = min(KG, K - k0);
   size_t r0 = rows * ch / nchunk, r1 = rows * (ch + 1) / nchunk;
@@ -88,6 +100,8 @@ __global__ void __launch_bounds__(kBlock, 2) k_multi_dot(const S* __restrict__ X
   const int q = warp_rows ? (tid & 31) % Q : tid % Q;
   const int lane = warp_rows ? (tid >> 5) * lw + wlane : tid / Q;
   const bool on = warp_rows ? wlane < lw : lane < lanes;
+  constexpr bool FLUSH = !PAIR;
+  static_assert(PAIR || VEC == 1, "lanes N <= kBlock");
   double are[FLUSH ? KG : 1][VEC], aim[FLUSH ? KG : 1][VEC];
   R pre[KG][VEC], pim[KG][VEC];
 #pragma unroll
@@ -128,7 +142,6 @@ __global__ void __launch_bounds__(kBlock, 2) k_multi_dot(const S* __restrict__ X
     }
   }
   if constexpr (FLUSH) {
-    static_assert(VEC == 1, "lanes * N <= kBlock");
 #pragma unroll
     for (int j = 0; j < KG; ++j)
       if (on && j < nk)
@@ -148,30 +161,61 @@ __global__ void __launch_bounds__(kBlock, 2) k_multi_dot(const S* __restrict__ X
       }
     for (int e = tid; e < nk * N; e += kBlock) res[e] = buf[(e / N) * kBlock + e % N];
   } else {
-    float2* wsum = reinterpret_cast<float2*>(buf);
-    const int units = warp_rows ? kBlock / 32 : lanes, unit = warp_rows ? tid >> 5 : lane;
+    float4* wsum = reinterpret_cast<float4*>(buf);  // (re hi, re lo, im hi, im lo)
+    constexpr int kWarps = kBlock / 32;
+    const int unit = tid >> 5;
     int half = 1;
     while (2 * half < lw) half *= 2;
+    if (lw == 1) half = 0;
 #pragma unroll
     for (int j = 0; j < KG; ++j) {
       if (j >= nk) break;
 #pragma unroll
       for (int e = 0; e < VEC; ++e) {
-        float a = pre[j][e], b = pim[j][e];
-        if (lw > 1)
-          for (int h = half; h > 0; h >>= 1) {
-            const float oa = __shfl_down_sync(0xffffffffu, a, h * Q), ob = __shfl_down_sync(0xffffffffu, b, h * Q);
-            if (wlane < h && wlane + h < lw) a += oa, b += ob;
-          }
-        if (on && wlane == 0) wsum[(j * units + unit) * N + VEC * q + e] = make_float2(a, b);
+        float a = pre[j][e], b = pim[j][e], al = 0.f, bl = 0.f;
+        for (int h = half; h > 0; h >>= 1) {
+          const float oa = __shfl_down_sync(0xffffffffu, a, h * Q), ob = __shfl_down_sync(0xffffffffu, b, h * Q);
+          float ol = 0.f, pl = 0.f;
+          if (h < half) ol = __shfl_down_sync(0xffffffffu, al, h * Q), pl = __shfl_down_sync(0xffffffffu, bl, h * Q);
+          if (wlane < h && wlane + h < lw) pair_add(a, al, oa, ol), pair_add(b, bl, ob, pl);
+        }
+        if (on && wlane == 0) wsum[(j * kWarps + unit) * N + VEC * q + e] = make_float4(a, al, b, bl);
       }
     }
     __syncthreads();
+    bool left = false;  // the range of FP32 (or the data are not finite)
     for (int e = tid; e < nk * N; e += kBlock) {
-      const float2* w = wsum + (size_t)(e / N) * units * N + e % N;
-      double2 t = make_double2(0, 0);
-      for (int u = 0; u < units; ++u) t.x += (double)w[u * N].x, t.y += (double)w[u * N].y;
-      res[e] = t;
+      const float4* w = wsum + (size_t)(e / N) * kWarps * N + e % N;
+      float4 t = w[0];
+#pragma unroll
+      for (int u = 1; u < kWarps; ++u) {
+        const float4 o = w[u * N];
+        pair_add(t.x, t.y, o.x, o.y), pair_add(t.z, t.w, o.z, o.w);
+      }
+      left = left || !isfinite(t.x) || !isfinite(t.z);
+      res[e] = make_double2((double)t.x + (double)t.y, (double)t.z + (double)t.w);
+    }
+    if (__syncthreads_or(left)) {
+#pragma unroll
+      for (int j = 0; j < KG; ++j) {
+        if (j >= nk) break;
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) {
+          double a = pre[j][e], b = pim[j][e];
+          for (int h = half; h > 0; h >>= 1) {
+            const double oa = __shfl_down_sync(0xffffffffu, a, h * Q), ob = __shfl_down_sync(0xffffffffu, b, h * Q);
+            if (wlane < h && wlane + h < lw) a += oa, b += ob;
+          }
+          if (on && wlane == 0) buf[unit * N + VEC * q + e] = make_double2(a, b);
+        }
+        __syncthreads();
+        for (int r = tid; r < N; r += kBlock) {
+          double2 t = buf[r];
+          for (int u = 1; u < kWarps; ++u) t.x += buf[u * N + r].x, t.y += buf[u * N + r].y;
+          res[j * N + r] = t;
+        }
+        __syncthreads();
+      }
     }
   }
   if (ranks > 1) cg::this_cluster().sync();
@@ -300,15 +344,6 @@ bool use_dot4(const void* X, size_t stride, const void* Y, int N, int dtype) {
 
 }  // namespace
 
-namespace {
-template <class S>
-auto dot_kernel(bool flush) {
-  if constexpr (sizeof(S) < 8)
-    if (!flush) return k_multi_dot<S, 1, kKG, false>;
-  return k_multi_dot<S, 1, kKG, true>;
-}
-}  // namespace
-
 size_t multi_dot_partials_bytes(size_t rows, int N, int K) {
   return sizeof(double) * 2 * (size_t)K * n_chunks(rows, N) * N;
 }
@@ -322,9 +357,10 @@ void multi_dot_ws(mrhs_ctx c, const void* X, size_t stride, int K, const void* Y
   // rows that a thread would sum with one CTA per chunk
   auto thread_rows = [&](int vec) { return (rows / nch) / dot_lanes(N / vec) + 1; };
   const bool four_ok = four && thread_rows(4) <= kMaxRows;
-  const int groups = (K + kKG - 1) / kKG;
+  const int kg = four_ok && N > kWide ? kKGWide : kKG;
+  const int groups = (K + kg - 1) / kg;
   const int ranks = nch * groups < kClusterBelow ? kClusterCtas : 1;
-  const bool flush = dtype == MRHS_F64 || thread_rows(1) > kMaxRows;
+  const bool one_ok = dtype == MRHS_F32 && N <= 32 && thread_rows(1) / ranks + 1 <= kFlush;
   Prof pr(c, "multi_dot");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nch * ranks, groups);
@@ -335,13 +371,16 @@ void multi_dot_ws(mrhs_ctx c, const void* X, size_t stride, int K, const void* Y
   at.val.clusterDim.x = ranks, at.val.clusterDim.y = 1, at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = ranks > 1 ? 1 : 0;
-  if (four_ok)
-    MRHS_CUDA(cudaLaunchKernelEx(&cfg, k_multi_dot<float, 4, kKG, false>, (const float*)X, stride, K, (const float*)Y,
-                                 rows, N, nch, ranks, part));
-  else
+  if (four_ok || one_ok) {
+    auto kern = !four_ok ? k_multi_dot<float, 1, kKG, true>
+                : kg == kKG ? k_multi_dot<float, 4, kKG, true> : k_multi_dot<float, 4, kKGWide, true>;
+    MRHS_CUDA(cudaLaunchKernelEx(&cfg, kern, (const float*)X, stride, K, (const float*)Y, rows, N, nch, ranks, part));
+  } else {
     MRHS_DISPATCH(dtype, S, {
-      MRHS_CUDA(cudaLaunchKernelEx(&cfg, dot_kernel<S>(flush), (const S*)X, stride, K, (const S*)Y, rows, N, nch, ranks, part));
+      MRHS_CUDA(cudaLaunchKernelEx(&cfg, k_multi_dot<S, 1, kKG, false>, (const S*)X, stride, K, (const S*)Y, rows, N, nch,
+                                   ranks, part));
     });
+  }
   MRHS_LAUNCH_CHECK("multi_dot");
   k_sum_chunks<<<grid_for((size_t)K * N * 32, 256), 256, 0, c->stream>>>(part, K, nch, N, out, out32);
   MRHS_LAUNCH_CHECK("sum_chunks");
