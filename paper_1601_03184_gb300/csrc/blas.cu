@@ -38,24 +38,22 @@ int n_chunks(size_t rows, int N) {
 // most kMaxRows or with VEC = 1 kFlush, in FP32, and the threads are joined, by shuffles
 // and then across the warps, in pairs of FP32 numbers (two-sums: 48 bits, where the rows'
 // own sums have 24); a pair that leaves the range of FP32 sends the CTA to the same joins
-// in FP64. (Over plain FP32 shuffles, five roundings more, the pairs cost 1 us of a call:
-// a coarse solve of 16^3 x 32 with 32 vectors takes 5.31 ms in place of 5.24.)
-// A chunk is one CTA, or a cluster of eight when the chunks alone would leave
-// most of the GPU idle: the ranks take eighths of the chunk and the first adds
-// their sums in order, so that the partials, and the workspace they need, stay
-// one per chunk.
+// in FP64. (Over plain FP32 shuffles, five roundings more, the pairs cost 1 us of a call
+// of 16384 x 32.)
+// A chunk is one CTA, or a cluster of two, four or eight while all CTAs still run
+// together, two to an SM: the ranks take equal parts of the chunk and the first adds their
+// sums in order, so that the partials, and the workspace they need, stay one per chunk.
+// More CTAs than that only repeat the joins: with clusters of eight below 304 CTAs
+// altogether (before) and by this rule, 152 SMs, per call: 1, 5, 10 and 20 vectors of 16384 x 32
+// 12.4, 20.6, 30.8, 53.7 -> 12.3, 16.5, 18.5, 28.7 us; of 12800 x 20 12.4, 16.5, 24.6, 38.8
+// -> 12.4, 16.5, 18.5, 30.8; of 98304 x 24 36, 96, 79, 146 -> 16, 53, 79, 145. 1 vector
+// of 4096 rows, one CTA a chunk and a serial FP64 sum: 97 us; now 10.
 constexpr int kKG = 4;          // vectors per group (its sums: up to 40 KB of shared memory)
 constexpr int kKGWide = 2;      // the same for VEC = 4 and more than kWide right-hand sides
 constexpr int kWide = 64;
 constexpr int kFlush = 32;
 constexpr int kMaxRows = 128;
 constexpr int kClusterCtas = 8;
-// CTAs (two for each of the 152 SMs) below which a chunk becomes a cluster.
-// Measured per call: 1 vector of 4096 rows, FP32 (one CTA and a serial FP64 sum
-// before) 97 -> 23 us; 1 to 20 vectors of 16384 x 32 (32 to 160 CTAs) 35 -> 28 us,
-// and 37 -> 20 us at 12800 x 20.
-constexpr int kClusterBelow = 304;
-
 template <class S, int VEC>
 __device__ __forceinline__ void ld_row(const S* p, typename Real<S>::type v[VEC]) {
   if constexpr (VEC == 4) {
@@ -359,7 +357,8 @@ void multi_dot_ws(mrhs_ctx c, const void* X, size_t stride, int K, const void* Y
   const bool four_ok = four && thread_rows(4) <= kMaxRows;
   const int kg = four_ok && N > kWide ? kKGWide : kKG;
   const int groups = (K + kg - 1) / kg;
-  const int ranks = nch * groups < kClusterBelow ? kClusterCtas : 1;
+  int ranks = kClusterCtas;
+  while (ranks > 1 && nch * groups * ranks > 2 * c->num_sms) ranks /= 2;
   const bool one_ok = dtype == MRHS_F32 && N <= 32 && thread_rows(1) / ranks + 1 <= kFlush;
   Prof pr(c, "multi_dot");
   cudaLaunchConfig_t cfg = {};

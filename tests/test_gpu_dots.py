@@ -38,12 +38,14 @@ def multi_dot(lat, X, Y, K, rows, N, dtype):
 # N = 1, 5, 33, 132: one right-hand side per thread, rows within a warp and across warps;
 # 4, 20, 64, 68, 128: four per thread, 16 rows each and, in the last two, the most (128,
 # with chunks capped) and one too many for them (one per thread again); few rows (clusters of
-# CTAs per chunk) and many (one CTA per chunk); one vector and a group with a remainder
+# eight CTAs per chunk), more (of four and of two) and many (one CTA per chunk); one vector
+# and a group with a remainder
 @pytest.mark.parametrize("N,rows,K,dtype", [
     (1, 4096, 5, MRHS_F32), (1, 5200000, 1, MRHS_F32), (5, 4100, 5, MRHS_F32), (5, 1100000, 1, MRHS_F32),
     (33, 4100, 5, MRHS_F32), (132, 4100, 2, MRHS_F32), (20, 4100, 5, MRHS_BF16), (5, 1100000, 1, MRHS_BF16),
     (5, 4100, 5, MRHS_F64), (4, 4100, 5, MRHS_F32), (20, 4100, 5, MRHS_F32), (20, 300000, 1, MRHS_F32),
     (64, 4100, 5, MRHS_F32), (68, 4100, 5, MRHS_F32), (128, 4100, 5, MRHS_F32),
+    (32, 16384, 5, MRHS_F32), (32, 16384, 10, MRHS_F32), (5, 105000, 5, MRHS_F32), (5, 105000, 10, MRHS_F32),
     (64, 2048 * 16 * 127, 1, MRHS_F32), (64, 2048 * 16 * 129, 1, MRHS_F32)])
 def test_whole_numbers(lat, N, rows, K, dtype):
     top = 255 if dtype == MRHS_BF16 or N % 4 == 0 and N <= 128 else 511
