@@ -233,12 +233,13 @@ __global__ void k_modrelu_back(const float* z, const float* dh, float* dz, const
 // and every G-th m, G = 256 / (4 x 4 tiles): eight 8-byte reads feed 64 FMAs, about
 // the balance of the two pipes. The FP32 sums run over at most kWgChain m and are
 // then added into (hi, lo) pairs (two-sum, 48 bits), FP64 being 1/64 of the FP32
-// rate here; the pairs of a tile's threads are joined in FP64 at the end.
+// rate here; the pairs of a tile's threads are joined in FP64 at the end. Where a sum left
+// the range of FP32 on the way, the CTA starts again with FP64 in place of the pairs (WIDE).
 // Before, a CTA staged 8 sites of one right-hand side at a time and each thread took
 // one (c, c') with two 8-byte reads and 3 FMAs per read: 2461 us a layer on average at
-// 16^4 sites, 8 right-hand sides, widths 4-11-11-4; now 1174 us (the loads of a tile in
+// 16^4 sites, 8 right-hand sides, widths 4-11-11-4; now 1225 us (the loads of a tile in
 // turn, then the joins at the end, are what is left).
-constexpr int kWgChain = 32;
+constexpr int kWgChain = 24;
 
 __device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
   const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
@@ -246,12 +247,29 @@ __device__ __forceinline__ void two_sum(float& hi, float& lo, float x) {
   hi = s;
 }
 
-__global__ void __launch_bounds__(256, 2) k_wgrad(const float* __restrict__ dz, const float* __restrict__ h,
-                                               const float* __restrict__ U32, const int* __restrict__ nbr, int cin,
-                                               int cout, int N, size_t V, size_t sites_per_cta, int cols,
-                                               double* part) {
+template <bool WIDE>
+struct WgSum;
+template <>
+struct WgSum<false> {
+  float hi[32], lo[32];
+  __device__ __forceinline__ void add(int e, float x) { two_sum(hi[e], lo[e], x); }
+  __device__ __forceinline__ double get(int e) const { return (double)hi[e] + (double)lo[e]; }
+  __device__ __forceinline__ void clear(int e) { hi[e] = lo[e] = 0.f; }
+};
+template <>
+struct WgSum<true> {
+  double v[32];
+  __device__ __forceinline__ void add(int e, float x) { v[e] += (double)x; }
+  __device__ __forceinline__ double get(int e) const { return v[e]; }
+  __device__ __forceinline__ void clear(int e) { v[e] = 0; }
+};
+
+// one CTA's partial sums; whether one that this thread wrote is not finite
+template <bool WIDE>
+__device__ __forceinline__ bool wgrad_cta(double* smem_wg, const float* __restrict__ dz, const float* __restrict__ h,
+                                          const float* __restrict__ U32, const int* __restrict__ nbr, int cin,
+                                          int cout, int N, size_t V, size_t sites_per_cta, int cols, double* part) {
   const int M = 3 * cols;
-  extern __shared__ double smem_wg[];
   float2* sdz = reinterpret_cast<float2*>(smem_wg);  // [4 ceil(cout/4)][M], the rows beyond cout zero
   const int nci = (cin + 3) / 4, nco = (cout + 3) / 4, ntile = nci * nco, G = 256 / ntile;
   float2* stv = sdz + 4 * nco * M;                // [4 ceil(cin/4)][M]
@@ -263,9 +281,10 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const float* __restrict__ dz, 
   const int g = tid % G, tile = tid / G;             // neighbouring lanes: neighbouring m
   const bool on = tile < ntile;
   const int c0 = 4 * (tile / nci), d0 = 4 * (tile % nci);
-  float acc[32], hi[32], lo[32];                     // [4][4][re, im]
+  float acc[32];                                     // [4][4][re, im]
+  WgSum<WIDE> tot;
 #pragma unroll
-  for (int e = 0; e < 32; ++e) acc[e] = hi[e] = lo[e] = 0.f;
+  for (int e = 0; e < 32; ++e) acc[e] = 0.f, tot.clear(e);
   for (int i = tid; i < 4 * (nco + nci) * M; i += 256) sdz[i] = make_float2(0.f, 0.f);
   __syncthreads();
   int chain = 0;
@@ -305,8 +324,10 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const float* __restrict__ dz, 
         }
       }
       __syncthreads();
-      if (on) {
-        for (int m = g; m < mm; m += G) {
+      for (int m = g; on && m < mm;) {
+        const int stop = min(mm, m + (kWgChain - chain) * G);
+        chain += (stop - m + G - 1) / G;
+        for (; m < stop; m += G) {
           float2 z[4], t[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) z[i] = sdz[(c0 + i) * M + m], t[i] = stv[(d0 + i) * M + m];
@@ -321,10 +342,9 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const float* __restrict__ dz, 
               im = fmaf(z[i].y, t[j].x, fmaf(-z[i].x, t[j].y, im));
             }
         }
-        chain += (mm + G - 1) / G;
-        if (chain + (M + G - 1) / G > kWgChain) {
+        if (chain == kWgChain) {
 #pragma unroll
-          for (int e = 0; e < 32; ++e) two_sum(hi[e], lo[e], acc[e]), acc[e] = 0.f;
+          for (int e = 0; e < 32; ++e) tot.add(e, acc[e]), acc[e] = 0.f;
           chain = 0;
         }
       }
@@ -332,19 +352,19 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const float* __restrict__ dz, 
     }
   }
 #pragma unroll
-  for (int e = 0; e < 32; ++e) two_sum(hi[e], lo[e], acc[e]);
+  for (int e = 0; e < 32; ++e) tot.add(e, acc[e]);
   // the G threads of a tile, eight entries at a time: four neighbouring threads sum a
   // quarter of them each and join by shuffles (a fixed order)
   double2* sum = reinterpret_cast<double2*>(smem_wg);  // [8][256]
   const int npair = cout * cin;
+  bool left = false;
 #pragma unroll
   for (int half = 0; half < 2; ++half) {
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const int i = 8 * half + e;
-      sum[e * 256 + tid] =
-          make_double2((double)hi[2 * i] + (double)lo[2 * i], (double)hi[2 * i + 1] + (double)lo[2 * i + 1]);
+      sum[e * 256 + tid] = make_double2(tot.get(2 * i), tot.get(2 * i + 1));
     }
     __syncthreads();
     for (int w = tid; w < ntile * 32; w += 256) {  // a warp per tile
@@ -364,9 +384,20 @@ __global__ void __launch_bounds__(256, 2) k_wgrad(const float* __restrict__ dz, 
         double* o = part + (((size_t)k * gridDim.y + blockIdx.y) * npair + c * cin + cp) * 2;
         o[0] = s.x;
         o[1] = s.y;
+        left = left || !isfinite(s.x) || !isfinite(s.y);
       }
     }
   }
+  return left;
+}
+
+__global__ void __launch_bounds__(256, 2) k_wgrad(const float* __restrict__ dz, const float* __restrict__ h,
+                                                  const float* __restrict__ U32, const int* __restrict__ nbr, int cin,
+                                                  int cout, int N, size_t V, size_t sites_per_cta, int cols,
+                                                  double* part) {
+  extern __shared__ double smem_wg[];
+  if (__syncthreads_or(wgrad_cta<false>(smem_wg, dz, h, U32, nbr, cin, cout, N, V, sites_per_cta, cols, part)))
+    wgrad_cta<true>(smem_wg, dz, h, U32, nbr, cin, cout, N, V, sites_per_cta, cols, part);
 }
 
 // G[k][p] += factor * sum of the per-CTA partials: a warp per (k, p), its lanes the
