@@ -512,6 +512,27 @@ __global__ void __launch_bounds__(kThreads, 2) k_coarse_op_tc(const SP* __restri
 // waited for; two CTAs share an SM.
 constexpr int kDcThreads = 512;  // 16 warps: the operand conversion is the CUDA cores' share
 
+// Part p of row i of aggregate A for right-hand side r in plain FP32. The low part of an
+// infinite operand (or of one that tf32 rounds to infinity) is not a number: where the split
+// products are not finite the sum is taken again, so that it is what the operands make it.
+__device__ __noinline__ float dc_plain(const float* __restrict__ Dc, const float* __restrict__ x0,
+                                       const float* __restrict__ xh, const int* __restrict__ aggnbr,
+                                       const int* __restrict__ pos, int A, int nc, int nrhs, int kb, int ke, int i,
+                                       int p, int r) {
+  float s = 0.f;
+  for (int k = kb; k < ke; ++k) {
+    const int B = k == 0 ? A : aggnbr[A * 8 + k - 1];
+    const float* xs = (k == 0 ? x0 : xh) + (size_t)(pos ? pos[B] : B) * nc * 2 * nrhs + r;
+    const float* d = Dc + (((size_t)A * 9 + k) * nc + i) * nc * 2;
+    for (int col = 0; col < nc; ++col) {
+      const float xr = xs[2 * col * nrhs], xi = xs[(2 * col + 1) * nrhs];
+      s = p == 0 ? fmaf(-d[2 * col + 1], xi, fmaf(d[2 * col], xr, s))
+                 : fmaf(d[2 * col + 1], xr, fmaf(d[2 * col], xi, s));
+    }
+  }
+  return s;
+}
+
 // A part of the stencil (the even-odd coarse solve): CTA b takes aggregate
 // alist[b] (b without a list) and the blocks kb <= k < ke; block 0 reads x0,
 // the hop blocks xh, the row block of aggregate B at pos[B] (B without pos);
@@ -524,7 +545,8 @@ __global__ void __launch_bounds__(kDcThreads, 1) k_apply_dc_tc(const float* __re
                                                                uint32_t tm_cols, int* __restrict__ err,
                                                                const int* __restrict__ alist,
                                                                const int* __restrict__ pos, int kb, int ke,
-                                                               const float* __restrict__ add) {
+                                                               const float* __restrict__ add,
+                                                               const float* __restrict__ Dfull) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint64_t full[2], mma_done;
   __shared__ uint32_t s_tmem;
@@ -717,13 +739,21 @@ __global__ void __launch_bounds__(kDcThreads, 1) k_apply_dc_tc(const float* __re
     __syncthreads();
     float* yA = y + (size_t)blockIdx.x * nc * 2 * nrhs;
     const float* addA = add ? add + (size_t)blockIdx.x * nc * 2 * nrhs : nullptr;
+    bool bad = false;
     for (int e = tid; e < nc * 2 * nrhs; e += kDcThreads) {
       const int r = e % nrhs, p = (e / nrhs) % 2, i = e / (2 * nrhs);
       float v = p == 0 ? E[i * (NM + 1) + r] - E[(nc + i) * (NM + 1) + nrhs + r]
                        : E[i * (NM + 1) + nrhs + r] + E[(nc + i) * (NM + 1) + r];
       if (addA) v += addA[e];
+      bad = bad || !isfinite(v);
       yA[e] = v;
     }
+    if (SPLIT && bad)
+      for (int e = tid; e < nc * 2 * nrhs; e += kDcThreads) {
+        if (isfinite(yA[e])) continue;
+        const float v = dc_plain(Dfull, x0, xh, aggnbr, pos, A, nc, nrhs, kb, ke, e / (2 * nrhs), e / nrhs % 2, e % nrhs);
+        yA[e] = addA ? v + addA[e] : v;
+      }
   } else {
     // a wait ran out: let the copies still in flight land before the CTA's
     // shared memory is released
@@ -889,7 +919,7 @@ bool apply_Dc_tc(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, bool split) {
   MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<pt.na, kDcThreads, smem, c->stream>>>((const float*)src, (const float*)pt.x0, (const float*)pt.xh,
                                                (float*)yc, c->aggnbr, nc, nrhs, cols, err, pt.alist, pt.pos, pt.kb,
-                                               pt.ke, (const float*)pt.add);
+                                               pt.ke, (const float*)pt.add, (const float*)c->Dc);
   MRHS_LAUNCH_CHECK("apply_dc_tc");
   return true;
 }
