@@ -11,13 +11,6 @@ namespace mrhs {
 namespace {
 
 constexpr int kSites = 8;  // sites staged per chunk in the contractions
-// Right-hand sides up to which the coarse stencil takes a warp per row
-// (k_apply_dc_rows). One thread per (eight rows, right-hand side) leaves the
-// GPU idle at few of them: 1 right-hand side, 512 aggregates, 2ntv = 40, FP32:
-// 397 -> 21 us per application; 4: 132 -> 36; 8: 119 -> 72 (the whole call; at
-// 4096 aggregates, 2ntv = 48: 890 -> 173, 675 -> 308, 760 -> 636 us). From 9 on
-// the row's registers would be read for a second group of vectors.
-constexpr int kRowsMaxRhs = 8;
 
 // One CTA per (aggregate A, stencil entry k). Columns (h', j), rows (h, i):
 //   k = 0:      sum_{x in A} P_(h,i)(x)^dag [A(x) + hops inside A] P_(h',j)
@@ -1162,16 +1155,13 @@ void apply_Dc_part(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, int dtype) 
   MRHS_REQUIRE(c->have_Dc, MRHS_ERR_STATE, "D_c used before mrhs_build_Dc");
   MRHS_REQUIRE(dtype == c->work_dtype, MRHS_ERR_ARG, "D_c apply: dtype must be the context's work type");
   const int nc = 2 * c->ntv;
-  // tensor cores unless the CUDA-core engine is chosen: split tf32 (FP32
-  // accuracy) for the FP32 setup, single tf32 for the mixed ones
+  // tensor cores unless the CUDA-core engine is chosen
   static const bool apply_alu = [] {
     const char* e = std::getenv("MRHS_DC_APPLY");
     return e && std::string(e) == "alu";
   }();
-  // (the mixed setups' other counts of right-hand sides keep FP32 accuracy: split)
   if (c->dc_engine != MRHS_DC_ALU && dtype == MRHS_F32 && !apply_alu && nrhs > kRowsMaxRhs) {
-    const bool split = c->prec == MRHS_PREC_FP32 || nrhs % 16 != 0;
-    if (apply_Dc_tc(c, pt, yc, nrhs, split)) return;
+    if (apply_Dc_tc(c, pt, yc, nrhs, dc_split(c, nrhs))) return;
   }
   Prof pr(c, "apply_dc");
   auto launch = [&](auto* tag) {

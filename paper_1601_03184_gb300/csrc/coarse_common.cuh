@@ -9,6 +9,14 @@ struct Agg4 {
   int a[4];
 };
 
+// Right-hand sides up to which the coarse stencil takes a warp per row
+// (k_apply_dc_rows). One thread per (eight rows, right-hand side) leaves the
+// GPU idle at few of them: 1 right-hand side, 512 aggregates, 2ntv = 40, FP32:
+// 397 -> 21 us per application; 4: 132 -> 36; 8: 119 -> 72 (the whole call; at
+// 4096 aggregates, 2ntv = 48: 890 -> 173, 675 -> 308, 760 -> 636 us). From 9 on
+// the row's registers would be read for a second group of vectors.
+constexpr int kRowsMaxRhs = 8;
+
 // local site index of face site f of an aggregate: l_mu fixed to lmu, the
 // other three coordinates enumerated lexicographically
 static __device__ __forceinline__ int face_site(const Agg4& g, int mu, int lmu, int f) {

@@ -546,7 +546,8 @@ __global__ void __launch_bounds__(kDcThreads, 1) k_apply_dc_tc(const float* __re
                                                                const int* __restrict__ alist,
                                                                const int* __restrict__ pos, int kb, int ke,
                                                                const float* __restrict__ add,
-                                                               const float* __restrict__ Dfull) {
+                                                               const float* __restrict__ Dfull,
+                                                               uint32_t img_pitch) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint64_t full[2], mma_done;
   __shared__ uint32_t s_tmem;
@@ -560,7 +561,8 @@ __global__ void __launch_bounds__(kDcThreads, 1) k_apply_dc_tc(const float* __re
   const int b_bytes = NM / 8 * KG * 128;     // B tile
   const uint32_t d_bytes = (uint32_t)nc * nc * 8, x_bytes = (uint32_t)nc * 2 * nrhs * 4;
   // PRE: the stage holds the block's ready operand images (hi, then lo) in
-  // place of the FP32 block, and the MMAs read A from the stage itself
+  // place of the FP32 block, and the MMAs read A from the stage itself; the images of
+  // consecutive blocks are img_pitch bytes apart (without SPLIT the hi image of a pair will do)
   const uint32_t img_bytes = (SPLIT ? 2 : 1) * (uint32_t)a_bytes;
   const uint32_t x_off = PRE ? img_bytes : d_bytes;  // the x block inside a stage
   const uint32_t raw_bytes = (x_off + x_bytes + 1023) & ~1023u;
@@ -627,7 +629,7 @@ __global__ void __launch_bounds__(kDcThreads, 1) k_apply_dc_tc(const float* __re
     const int rb = pos ? pos[B] : B;
     tc::mbar_expect_tx(&full[j & 1], x_off + x_bytes);
     if (PRE)
-      tc::bulk_g2s(raw, reinterpret_cast<const unsigned char*>(Dc) + ((size_t)A * 9 + k) * img_bytes, img_bytes,
+      tc::bulk_g2s(raw, reinterpret_cast<const unsigned char*>(Dc) + ((size_t)A * 9 + k) * img_pitch, img_bytes,
                    &full[j & 1]);
     else
       tc::bulk_g2s(raw, Dc + ((size_t)A * 9 + k) * nc * nc * 2, d_bytes, &full[j & 1]);
@@ -836,9 +838,15 @@ bool build_Dc_tc(mrhs_ctx c, int fmt, bool split) {
   return true;
 }
 
+// The form of the tensor-core coarse stencil for nrhs right-hand sides: split tf32, or in the
+// mixed setups single tf32 for a multiple of 16 (the other counts, CUDA-core ones by origin,
+// keep FP32 accuracy)
+bool dc_split(mrhs_ctx c, int nrhs) { return c->prec == MRHS_PREC_FP32 || nrhs % 16 != 0; }
+
 // the operand images of D_c for the tensor-core coarse stencil, made by every
 // build of D_c (so that the coarse solves, including the allocation-free one,
-// only read them): tf32 hi + lo for the FP32 setup, tf32 for the mixed ones.
+// only read them): tf32 hi + lo for the FP32 setup and for the mixed ones whose vectors
+// take the split form, tf32 for the others.
 // Skipped (the stencil then converts each block itself) when the stencil
 // would not use them, when MRHS_DC_IMAGES=0, or when they do not fit in
 // device memory.
@@ -850,7 +858,8 @@ void dc_images_build(mrhs_ctx c) {
   }();
   const int nc = 2 * c->ntv, KG = nc / 4;
   if (off || c->dc_engine == MRHS_DC_ALU || c->work_dtype != MRHS_F32 || nc % 8 != 0 || nc > 64) return;
-  const bool split = c->prec == MRHS_PREC_FP32;
+  const int nb = c->block_len > 0 ? std::min(c->block_len, c->ntv) : c->ntv;  // vectors of the setup's solves
+  const bool split = dc_split(c, nb > kRowsMaxRhs ? nb : 16);  // fewer vectors never take this form
   const size_t a_bytes = (size_t)kRows / 8 * KG * 128;
   const size_t nblk = (size_t)c->g.nagg * 9;
   if (!c->dc_img) {
@@ -880,7 +889,8 @@ void dc_images_build(mrhs_ctx c) {
 // of right-hand sides from 9 on (the columns are filled up to 16 with zeros): at
 // 16^3x32, 2ntv = 40, 20 of them take 73 us against 114 on the CUDA cores, 9 take 67
 // against 126; in the even-odd solve 41 us a launch against 109; 32^3x64, bf16
-// setup, 24 (split, converting each block): 1.24 against 1.85 ms
+// setup, 24 (split, converting each block): 1.24 against 1.85 ms; from images 15 % less (32^4:
+// 636 -> 539 us, and the single form from the same images 16: 365 -> 366, 32: 420 -> 420)
 bool apply_Dc_tc(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, bool split) {
   const int nc = 2 * c->ntv;
   if (c->work_dtype != MRHS_F32 || nc % 8 != 0 || nc > 64 || nrhs > 64) return false;
@@ -895,7 +905,7 @@ bool apply_Dc_tc(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, bool split) {
   while (cols < (uint32_t)(2 * NM)) cols <<= 1;  // R and S regions of NM columns each
   int* err = c->dflag + 3;
   const void* src = c->Dc;
-  bool pre = c->dc_img && c->dc_img_version == c->dc_version && c->dc_img_split == (int)split;
+  bool pre = c->dc_img && c->dc_img_version == c->dc_version && c->dc_img_split >= (int)split;
   // A recorded call is replayed on the D_c of the moment, which the images hold only as
   // long as every build makes them (not after a change of engine): counts that are not a
   // multiple of 16 read D_c itself, as they did on the CUDA cores.
@@ -919,7 +929,8 @@ bool apply_Dc_tc(mrhs_ctx c, const DcPart& pt, void* yc, int nrhs, bool split) {
   MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<pt.na, kDcThreads, smem, c->stream>>>((const float*)src, (const float*)pt.x0, (const float*)pt.xh,
                                                (float*)yc, c->aggnbr, nc, nrhs, cols, err, pt.alist, pt.pos, pt.kb,
-                                               pt.ke, (const float*)pt.add, (const float*)c->Dc);
+                                               pt.ke, (const float*)pt.add, (const float*)c->Dc,
+                                               (uint32_t)((c->dc_img_split ? 2 : 1) * (kRows / 8 * KG * 128)));
   MRHS_LAUNCH_CHECK("apply_dc_tc");
   return true;
 }

@@ -344,6 +344,7 @@ void apply_Dc_part(mrhs_ctx c, const DcPart& part, void* yc, int nrhs, int dtype
 bool covconv_tc(mrhs_ctx c, const float* h, float* z, const float* W, int cin, int cout, int N);
 void check_nn_tc_timeout(mrhs_ctx c);
 void dc_images_build(mrhs_ctx c);
+bool dc_split(mrhs_ctx c, int nrhs);
 void check_tc_timeout(mrhs_ctx c);
 void restrict_(mrhs_ctx c, const void* v, void* vc, int nrhs, int dtype);
 void prolong(mrhs_ctx c, const void* uc, void* u, int nrhs, int dtype);
