@@ -1525,8 +1525,6 @@ static void coarse_gmres(mrhs_ctx c, const void* bc, void* xc, int N, int dtype,
   };
   // the counts of the right-hand sides that go on: one pinned word and one
   // event per step, two of each in turn
-  for (auto& e : c->gm_event)
-    if (!e) MRHS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   int* hcount = c->hflag + 8;
   const bool ahead = fe * es <= kRunAheadBytes;
   int marks = 0;  // counts asked for so far

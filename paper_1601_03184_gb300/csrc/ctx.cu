@@ -770,6 +770,7 @@ int mrhs_create(const int dims[4], const int agg[4], int ntv, int prec, void* st
       c->dflag = (int*)dalloc(c, sizeof(int) * 16);
       c->coef32 = (float*)dalloc(c, sizeof(float) * 65 * 256 * 2);
       MRHS_CUDA(cudaMallocHost((void**)&c->hflag, sizeof(int) * 16));
+      for (auto& e : c->gm_event) MRHS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
       GeomArgs ga = geom_args(g);
       k_tables<<<grid_for(V, 256), 256, 0, c->stream>>>(ga, c->nbr, c->perm, c->iperm);
       MRHS_LAUNCH_CHECK("tables");
