@@ -655,6 +655,55 @@ __global__ void k_prolong6(const SP* __restrict__ P, const SC* __restrict__ uc, 
   for (int cc = 0; cc < 6; ++cc) st<SU, R>(u, s * 12 + 6 * h + cc, N, r, acc[cc]);
 }
 
+// The same for FP32 fields with N % 4 == 0 and an odd count of at most kProNarrow vectors:
+// four right-hand sides per thread (16-byte loads of uc and stores of u), one site's six rows
+// of P, so that every P entry loaded serves 4 x 6 complex products. More vectors, or an even
+// count, take the tiles below, whose rows need wider loads or more columns to pay: 16^4, FP32,
+// 4, 8, 16 and 24 right-hand sides, this form and the tiles: 5 vectors 23, 23, 37, 51 and 23, 27,
+// 42, 54 us; 7: 35, 33, 47, 64 and 29, 33, 49, 64; 9: 60, 43, 58, 76 and 33, 39, 55, 71; bf16 P, 5: 21,
+// 23, 37, 52 and 21, 24, 39, 52; 7: 25, 27, 45, 62 and 26, 29, 46, 62; 9: 31, 33, 54, 74 and 31, 35,
+// 52, 68.
+constexpr int kProNarrow = 7;
+template <class SP>
+__global__ void k_prolong6x4(const SP* __restrict__ P, const float* __restrict__ uc, float* __restrict__ u, int Nt,
+                             int N, int Va, size_t nwork) {
+  const int Q = N / 4;
+  const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (t >= nwork) return;
+  const int r0 = 4 * (int)(t % Q);
+  const size_t q = t / Q;
+  const int h = (int)(q % 2);
+  const size_t s = q / 2;
+  const size_t A = s / Va;
+  float are[6][4], aim[6][4];
+#pragma unroll
+  for (int cc = 0; cc < 6; ++cc)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) are[cc][e] = aim[cc][e] = 0.f;
+  for (int j = 0; j < Nt; ++j) {
+    const size_t crow = A * 2 * Nt + h * Nt + j;
+    const float4 w0 = *reinterpret_cast<const float4*>(uc + fidx(crow, 0, N, r0));
+    const float4 w1 = *reinterpret_cast<const float4*>(uc + fidx(crow, 1, N, r0));
+    const float wr[4] = {w0.x, w0.y, w0.z, w0.w}, wi[4] = {w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+    for (int cc = 0; cc < 6; ++cc) {
+      const cx<float> pv = ld<SP, float>(P, s * 12 + 6 * h + cc, Nt, j);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        // fma_(acc, p, w): acc.re += p.re w.re - p.im w.im, acc.im += p.re w.im + p.im w.re
+        are[cc][e] = fmaf(-pv.im, wi[e], fmaf(pv.re, wr[e], are[cc][e]));
+        aim[cc][e] = fmaf(pv.im, wr[e], fmaf(pv.re, wi[e], aim[cc][e]));
+      }
+    }
+  }
+#pragma unroll
+  for (int cc = 0; cc < 6; ++cc) {
+    const size_t row = s * 12 + 6 * h + cc;
+    *reinterpret_cast<float4*>(u + fidx(row, 0, N, r0)) = make_float4(are[cc][0], are[cc][1], are[cc][2], are[cc][3]);
+    *reinterpret_cast<float4*>(u + fidx(row, 1, N, r0)) = make_float4(aim[cc][0], aim[cc][1], aim[cc][2], aim[cc][3]);
+  }
+}
+
 // W consecutive values of a row in FP32, W 4, 2 or 1
 template <int W, class S>
 __device__ __forceinline__ void ld_some(const S* p, float* v) {
@@ -683,8 +732,8 @@ __device__ __forceinline__ void ld_some(const S* p, float* v) {
 // aggregates, 32 x 32, FP32: 514 -> 326 us; 8192, 24 x 24, bf16 P: 4822 -> 3112 us.
 // W: columns of P in one load, the largest of 4, 2 and 1 that divides Nt (a row
 // starts on a multiple of W only then); W = 1 still takes four columns a step. 16^4,
-// FP32, before (a thread with one site's six rows) and after: 13 x 8 63 -> 54 us,
-// 13 x 24 104 -> 90, 6 x 8 29 -> 28; bf16 P: 10 x 8 36 -> 32, 13 x 8 45 -> 48.
+// FP32, before (a thread with one site's six rows) and after: 13 x 8 63 -> 50 us,
+// 13 x 24 103 -> 89, 6 x 8 29 -> 27; bf16 P: 10 x 8 36 -> 32, 13 x 8 44 -> 44.
 constexpr int kProRows = 4;
 template <class SP, int W>
 __global__ void __launch_bounds__(256) k_prolong_tile(const SP* __restrict__ P, const float* __restrict__ uc,
@@ -1099,13 +1148,22 @@ void prolong_typed(mrhs_ctx c, const void* uc, int dc, void* u, int du, int N) {
   size_t work = (size_t)c->g.V * 2 * N;
   Prof pr(c, "prolong");
   const bool aligned = ((uintptr_t)uc & 15) == 0 && ((uintptr_t)u & 15) == 0;
+  if (dc == MRHS_F32 && du == MRHS_F32 && N % 4 == 0 && aligned && c->ntv % 2 != 0 && c->ntv <= kProNarrow) {
+    const size_t w4 = (size_t)c->g.V * 2 * (N / 4);
+    MRHS_DISPATCH(c->tv_dtype, SP, (k_prolong6x4<SP><<<grid_for(w4, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, w4)));
+    MRHS_LAUNCH_CHECK("prolong6x4");
+    return;
+  }
   if (dc == MRHS_F32 && du == MRHS_F32 && N % 4 == 0 && aligned) {
     // the block's columns in pieces of at most 48 KB (Nt <= 64: 24 groups and more), and
-    // two rounds of a CTA's threads over its rows: the coarse block staged serves them
+    // at most two rounds of a CTA's threads over its rows, which the staged block serves;
+    // one round where two CTAs do (16^4, 13 vectors, 4 right-hand sides: 47 -> 43 us). (A third
+    // round instead of another CTA, at 8 right-hand sides: 54 us against 50.)
     const int QC = std::min(N / 4, 48 * 1024 / (32 * c->ntv));
     const size_t smem = (size_t)32 * c->ntv * QC;
     const int tiles = (6 * c->g.Va + kProRows - 1) / kProRows * QC, threads = std::min(256, (tiles + 31) / 32 * 32);
-    const dim3 grid(2 * c->g.nagg, std::max(1, tiles / 512), (N / 4 + QC - 1) / QC);
+    const int per = tiles <= 512 ? 256 : 512;
+    const dim3 grid(2 * c->g.nagg, (tiles + per - 1) / per, (N / 4 + QC - 1) / QC);
     MRHS_DISPATCH(c->tv_dtype, SP, {
       if (c->ntv % 4 == 0)
         k_prolong_tile<SP, 4><<<grid, threads, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, QC);
