@@ -298,15 +298,13 @@ __device__ __forceinline__ void ld_four(const S* p, float v[4]) {
   if constexpr (sizeof(S) == 4) {
     const float4 t = __ldg(reinterpret_cast<const float4*>(p));
     v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
-  } else if constexpr (sizeof(S) == 2) {
+  } else {
+    static_assert(sizeof(S) == 2, "FP32 or a 16-bit type");
     const uint2 t = __ldg(reinterpret_cast<const uint2*>(p));
     S h[4];
     *reinterpret_cast<uint2*>(h) = t;
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = to_r(h[i]);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = (float)p[i];
   }
 }
 
@@ -315,8 +313,8 @@ __device__ __forceinline__ void ld_four(const S* p, float v[4]) {
 // starts on 8 bytes)
 template <class S>
 __device__ __forceinline__ void cp_runs(S* dst, const S* src, int n, size_t pitch, int ns) {
-  constexpr int E = 8 / (int)sizeof(S) > 0 ? 8 / (int)sizeof(S) : 1, W = sizeof(S) == 4 ? 4 : E;
-  const int per = n / W;  // pieces of a run (16 bytes for FP32)
+  constexpr int W = 4;  // elements of a piece (16 bytes for FP32)
+  const int per = n / W;
   for (int i = threadIdx.x; i < ns * per; i += 256) {
     const int k = i / per, e = (i - k * per) * W;
     const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + k * n + e);
@@ -333,15 +331,13 @@ __device__ __forceinline__ void lds_four(const S* p, float v[4]) {
   if constexpr (sizeof(S) == 4) {
     const float4 t = *reinterpret_cast<const float4*>(p);
     v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
-  } else if constexpr (sizeof(S) == 2) {
+  } else {
+    static_assert(sizeof(S) == 2, "FP32 or a 16-bit type");
     const uint2 t = *reinterpret_cast<const uint2*>(p);
     S h[4];
     *reinterpret_cast<uint2*>(h) = t;
 #pragma unroll
     for (int i = 0; i < 4; ++i) v[i] = to_r(h[i]);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = (float)p[i];
   }
 }
 
@@ -1083,6 +1079,23 @@ void build_Dc(mrhs_ctx c) {
   dc_images_build(c);
 }
 
+// The type pairs that the transfer operators meet: P has the storage type of the setup,
+// fine and coarse fields the work type (FP64 in the FP64 setup, else FP32) or, the vectors
+// that a refinement restricts, P's own. f(P's type, the fine field's type, the coarse one's).
+template <class F>
+static void transfer_types(mrhs_ctx c, int dfine, int dcoarse, F&& f) {
+  MRHS_REQUIRE(dcoarse == c->work_dtype && (dfine == c->work_dtype || dfine == c->tv_dtype), MRHS_ERR_ARG,
+               "fields are of the context's work type");
+  const bool own = dfine != c->work_dtype;  // a reduced storage type
+  switch (c->tv_dtype) {
+    case MRHS_F64: return f((double*)0, (double*)0, (double*)0);
+    case MRHS_F32: return f((float*)0, (float*)0, (float*)0);
+    case MRHS_BF16:
+      return own ? f((__nv_bfloat16*)0, (__nv_bfloat16*)0, (float*)0) : f((__nv_bfloat16*)0, (float*)0, (float*)0);
+    default: return own ? f((__half*)0, (__half*)0, (float*)0) : f((__half*)0, (float*)0, (float*)0);
+  }
+}
+
 // restriction from a fine field of type dv into a coarse field of type dc
 void restrict_typed(mrhs_ctx c, const void* v, int dv, void* vc, int dc, int N) {
   MRHS_REQUIRE(c->have_P, MRHS_ERR_STATE, "restriction before mrhs_build_P");
@@ -1097,49 +1110,35 @@ void restrict_typed(mrhs_ctx c, const void* v, int dv, void* vc, int dc, int N) 
     return e && std::string(e) == "tiled";
   }();
   // (a caller's field that does not start on 16 bytes takes the forms without wide copies)
-  if (!split_off && dc == MRHS_F32 && ((uintptr_t)v & 15) == 0) {
-    const bool vp = Nt % 4 == 0, vv = N % 4 == 0;
-    MRHS_DISPATCH(c->tv_dtype, SP, MRHS_DISPATCH(dv, SV, {
-      auto kern = N <= 3 && vp ? k_restrict_split<SP, SV, 1, true, false>
-                  : N <= 3     ? k_restrict_split<SP, SV, 1, false, false>
-                  : vp && vv   ? k_restrict_split<SP, SV, 4, true, true>
-                               : k_restrict_split<SP, SV, 4, false, false>;
-      const size_t stage = 2 * (size_t)kResSites * 12;
-      const size_t smem = std::max((stage * Nt * sizeof(SP) + 15) / 16 * 16 + stage * N * sizeof(SV),
-                                   sizeof(float2) * 256 * 2 * (N <= 3 ? 1 : 4));
-      MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      kern<<<2 * c->g.nagg, 256, smem, c->stream>>>((const SP*)c->P, (const SV*)v, (float*)vc, Nt, N, c->g.Va);
-    }));
-    MRHS_LAUNCH_CHECK("restrict_split");
-    return;
-  }
-  const bool tiled = Nt % 4 == 0 && N % 2 == 0 && (nc / 4) * (N / 2) <= 256;
-  MRHS_DISPATCH(c->tv_dtype, SP, MRHS_DISPATCH(dv, SV, {
-    if (tiled) {
-      if (dc == MRHS_F64) {
-        size_t smem = sizeof(cx<double>) * kSites * 12 * (size_t)(Nt + N);
-        auto kern = k_restrict_tiled<SP, SV, double>;
+  transfer_types(c, dv, dc, [&](auto* tp, auto* tv, auto* tc) {
+    using SP = std::remove_pointer_t<decltype(tp)>;
+    using SV = std::remove_pointer_t<decltype(tv)>;
+    using SC = std::remove_pointer_t<decltype(tc)>;
+    using R = typename Real<SC>::type;
+    if constexpr (sizeof(SC) == 4) {
+      // (a caller's field that does not start on 16 bytes takes the forms without wide copies)
+      if (!split_off && ((uintptr_t)v & 15) == 0) {
+        const bool vp = Nt % 4 == 0, vv = N % 4 == 0;
+        auto kern = N <= 3 && vp ? k_restrict_split<SP, SV, 1, true, false>
+                    : N <= 3     ? k_restrict_split<SP, SV, 1, false, false>
+                    : vp && vv   ? k_restrict_split<SP, SV, 4, true, true>
+                                 : k_restrict_split<SP, SV, 4, false, false>;
+        const size_t stage = 2 * (size_t)kResSites * 12;
+        const size_t smem = std::max((stage * Nt * sizeof(SP) + 15) / 16 * 16 + stage * N * sizeof(SV),
+                                     sizeof(float2) * 256 * 2 * (N <= 3 ? 1 : 4));
         MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kern<<<c->g.nagg, 256, smem, c->stream>>>((const SP*)c->P, (const SV*)v, (double*)vc, Nt, N, c->g.Va);
-      } else {
-        size_t smem = sizeof(cx<float>) * kSites * 12 * (size_t)(Nt + N);
-        auto kern = k_restrict_tiled<SP, SV, float>;
-        MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kern<<<c->g.nagg, 256, smem, c->stream>>>((const SP*)c->P, (const SV*)v, (float*)vc, Nt, N, c->g.Va);
+        kern<<<2 * c->g.nagg, 256, smem, c->stream>>>((const SP*)c->P, (const SV*)v, (float*)vc, Nt, N, c->g.Va);
+        MRHS_LAUNCH_CHECK("restrict_split");
+        return;
       }
-    } else if (dc == MRHS_F64) {
-      size_t smem = sizeof(cx<double>) * kSites * 12 * (size_t)(Nt + N);
-      auto kern = k_restrict<SP, SV, double, 8>;
-      MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      kern<<<c->g.nagg, threads, smem, c->stream>>>((const SP*)c->P, (const SV*)v, (double*)vc, Nt, N, c->g.Va);
-    } else {
-      size_t smem = sizeof(cx<float>) * kSites * 12 * (size_t)(Nt + N);
-      auto kern = k_restrict<SP, SV, float, 8>;
-      MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      kern<<<c->g.nagg, threads, smem, c->stream>>>((const SP*)c->P, (const SV*)v, (float*)vc, Nt, N, c->g.Va);
     }
-  }));
-  MRHS_LAUNCH_CHECK("restrict");
+    const bool tiled = Nt % 4 == 0 && N % 2 == 0 && (nc / 4) * (N / 2) <= 256;
+    const size_t smem = sizeof(cx<R>) * kSites * 12 * (size_t)(Nt + N);
+    auto kern = tiled ? k_restrict_tiled<SP, SV, SC> : k_restrict<SP, SV, SC, 8>;
+    MRHS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kern<<<c->g.nagg, tiled ? 256 : threads, smem, c->stream>>>((const SP*)c->P, (const SV*)v, (SC*)vc, Nt, N, c->g.Va);
+    MRHS_LAUNCH_CHECK("restrict");
+  });
 }
 
 void prolong_typed(mrhs_ctx c, const void* uc, int dc, void* u, int du, int N) {
@@ -1148,51 +1147,51 @@ void prolong_typed(mrhs_ctx c, const void* uc, int dc, void* u, int du, int N) {
   size_t work = (size_t)c->g.V * 2 * N;
   Prof pr(c, "prolong");
   const bool aligned = ((uintptr_t)uc & 15) == 0 && ((uintptr_t)u & 15) == 0;
-  if (dc == MRHS_F32 && du == MRHS_F32 && N % 4 == 0 && aligned && c->ntv % 2 != 0 && c->ntv <= kProNarrow) {
-    const size_t w4 = (size_t)c->g.V * 2 * (N / 4);
-    MRHS_DISPATCH(c->tv_dtype, SP, (k_prolong6x4<SP><<<grid_for(w4, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, w4)));
-    MRHS_LAUNCH_CHECK("prolong6x4");
-    return;
-  }
-  if (dc == MRHS_F32 && du == MRHS_F32 && N % 4 == 0 && aligned) {
-    // the block's columns in pieces of at most 48 KB (Nt <= 64: 24 groups and more), and
-    // at most two rounds of a CTA's threads over its rows, which the staged block serves;
-    // one round where two CTAs do (16^4, 13 vectors, 4 right-hand sides: 47 -> 43 us). (A third
-    // round instead of another CTA, at 8 right-hand sides: 54 us against 50.)
-    const int QC = std::min(N / 4, 48 * 1024 / (32 * c->ntv));
-    const size_t smem = (size_t)32 * c->ntv * QC;
-    const int tiles = (6 * c->g.Va + kProRows - 1) / kProRows * QC, threads = std::min(256, (tiles + 31) / 32 * 32);
-    const int per = tiles <= 512 ? 256 : 512;
-    const dim3 grid(2 * c->g.nagg, (tiles + per - 1) / per, (N / 4 + QC - 1) / QC);
-    MRHS_DISPATCH(c->tv_dtype, SP, {
-      if (c->ntv % 4 == 0)
-        k_prolong_tile<SP, 4><<<grid, threads, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, QC);
-      else if (c->ntv % 2 == 0)
-        k_prolong_tile<SP, 2><<<grid, threads, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, QC);
-      else
-        k_prolong_tile<SP, 1><<<grid, threads, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, QC);
-    });
-    MRHS_LAUNCH_CHECK("prolong_tile");
-    return;
-  }
-  if (dc == MRHS_F32 && du == MRHS_F32 && c->ntv % 4 == 0 && N == 1 && aligned) {
-    const size_t nrow = (size_t)c->g.V * 12;
-    MRHS_DISPATCH(c->tv_dtype, SP, {
-      if (c->ntv <= 16)
-        k_prolong_one<SP, 4><<<grid_for(nrow * 4, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, c->g.Va, nrow);
-      else
-        k_prolong_one<SP, 8><<<grid_for(nrow * 8, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, c->g.Va, nrow);
-    });
-    MRHS_LAUNCH_CHECK("prolong_one");
-    return;
-  }
-  MRHS_DISPATCH(c->tv_dtype, SP, MRHS_DISPATCH(du, SU, {
-    if (dc == MRHS_F64)
-      k_prolong6<SP, double, SU><<<grid_for(work, 256), 256, 0, c->stream>>>((const SP*)c->P, (const double*)uc, (SU*)u, c->ntv, N, c->g.Va, work);
-    else
-      k_prolong6<SP, float, SU><<<grid_for(work, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (SU*)u, c->ntv, N, c->g.Va, work);
-  }));
-  MRHS_LAUNCH_CHECK("prolong");
+  transfer_types(c, du, dc, [&](auto* tp, auto* tu, auto* tc) {
+    using SP = std::remove_pointer_t<decltype(tp)>;
+    using SU = std::remove_pointer_t<decltype(tu)>;
+    using SC = std::remove_pointer_t<decltype(tc)>;
+    if constexpr (std::is_same_v<SU, SC>) {
+      if constexpr (sizeof(SC) == 4) {
+        if (N % 4 == 0 && aligned && c->ntv % 2 != 0 && c->ntv <= kProNarrow) {
+          const size_t w4 = (size_t)c->g.V * 2 * (N / 4);
+          k_prolong6x4<SP><<<grid_for(w4, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N,
+                                                                     c->g.Va, w4);
+          MRHS_LAUNCH_CHECK("prolong6x4");
+          return;
+        }
+        if (N % 4 == 0 && aligned) {
+          // the block's columns in pieces of at most 48 KB (Nt <= 64: 24 groups and more), and
+          // at most two rounds of a CTA's threads over its rows, which the staged block serves;
+          // one round where two CTAs do (16^4, 13 vectors, 4 right-hand sides: 47 -> 43 us). (A
+          // third round instead of another CTA, at 8 right-hand sides: 54 us against 50.)
+          const int QC = std::min(N / 4, 48 * 1024 / (32 * c->ntv));
+          const size_t smem = (size_t)32 * c->ntv * QC;
+          const int tiles = (6 * c->g.Va + kProRows - 1) / kProRows * QC, threads = std::min(256, (tiles + 31) / 32 * 32);
+          const int per = tiles <= 512 ? 256 : 512;
+          const dim3 grid(2 * c->g.nagg, (tiles + per - 1) / per, (N / 4 + QC - 1) / QC);
+          auto kern = c->ntv % 4 == 0 ? k_prolong_tile<SP, 4> : c->ntv % 2 == 0 ? k_prolong_tile<SP, 2> : k_prolong_tile<SP, 1>;
+          kern<<<grid, threads, smem, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, N, c->g.Va, QC);
+          MRHS_LAUNCH_CHECK("prolong_tile");
+          return;
+        }
+        if (c->ntv % 4 == 0 && N == 1 && aligned) {
+          const size_t nrow = (size_t)c->g.V * 12;
+          const int lpr = c->ntv <= 16 ? 4 : 8;
+          auto kern = lpr == 4 ? k_prolong_one<SP, 4> : k_prolong_one<SP, 8>;
+          kern<<<grid_for(nrow * lpr, 256), 256, 0, c->stream>>>((const SP*)c->P, (const float*)uc, (float*)u, c->ntv, c->g.Va,
+                                                                 nrow);
+          MRHS_LAUNCH_CHECK("prolong_one");
+          return;
+        }
+      }
+      k_prolong6<SP, SC, SU><<<grid_for(work, 256), 256, 0, c->stream>>>((const SP*)c->P, (const SC*)uc, (SU*)u, c->ntv, N,
+                                                                         c->g.Va, work);
+      MRHS_LAUNCH_CHECK("prolong");
+    } else {
+      MRHS_REQUIRE(false, MRHS_ERR_ARG, "prolongation: fine fields are of the context's work type");
+    }
+  });
 }
 
 void restrict_(mrhs_ctx c, const void* v, void* vc, int nrhs, int dtype) {
