@@ -166,8 +166,8 @@ int mrhs_apply_D_block(mrhs_ctx ctx, const void* x, void* y, int nrhs, int dtype
  * FP32 fields on domains of 129 to 256 sites, nrhs a multiple of 4 and at
  * least two sweeps: works on copies of b and x (and of the links: 320 bytes a
  * site) in a workspace of at most 20 GB (or MRHS_TILE_BYTES, when that is in
- * the environment of mrhs_create) and a quarter of the free memory, taken for
- * the length of the call and given back in stream order to a memory pool of
+ * the environment of mrhs_create) and 3/4 of the free memory, taken for the
+ * length of the call and given back in stream order to a memory pool of
  * the context. The pool keeps it until mrhs_trim or mrhs_destroy, unless a
  * cudaMalloc of the process needs it: the driver then takes what is idle.
  * Without room for it the same smoother runs on the fields themselves. So does

@@ -1028,7 +1028,7 @@ static SapGeo sap_face_geo(mrhs_ctx c, int T, size_t* smem) {
 }
 
 // Right-hand sides smoothed together on tile copies: all of them when the workspace (the
-// links and two copies) takes at most tile_limit bytes (20 GB; or a quarter of what is free), else fewer, so
+// links and two copies) takes at most tile_limit bytes (20 GB; or 3/4 of what is free), else fewer, so
 // that the largest lattices keep their memory for the setup, in multiples of 8: of a row's
 // 128 bytes (32 right-hand sides) whole 64-byte pieces come from memory, so copies of four
 // at a time cost as much as of eight (48^3 x 96, 32 vectors, a setup: 545 ms in fours,
@@ -1043,7 +1043,7 @@ static int sap_group(mrhs_ctx c, int nrhs, size_t links) {
     const Unrecorded u;
     size_t free_b = 0, total_b = 0;
     MRHS_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    room = std::max(held, std::min(room, (free_b + held) / 4));
+    room = std::max(held, std::min(room, (free_b + held) / 4 * 3));
   }
   if (room < links + four) return 0;
   const int group = std::min(kTileGroup, 4 * (int)std::min<size_t>(nrhs / 4, (room - links) / four));
