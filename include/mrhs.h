@@ -245,10 +245,11 @@ int mrhs_restrict(mrhs_ctx ctx, const void* v, void* vc, int nrhs, int dtype);
 /* prolongation u = P uc (Sec. 2, Algorithm 1) */
 int mrhs_prolong(mrhs_ctx ctx, const void* uc, void* u, int nrhs, int dtype);
 /* yc = D_c xc on nrhs coarse right-hand sides (Sec. 5: D_c applied with the
- * same broadcast scheme as the restriction). With F32 coarse fields, 9 <= nrhs <=
- * 64, 2*ntv a multiple of 8 up to 64 (from 16 on unless 16 divides nrhs), an engine other than MRHS_DC_ALU and
- * pipeline stages that fit in shared memory (the split form at 2*ntv = 64
- * takes up to 48 right-hand sides) the products run on the tensor cores
+ * same broadcast scheme as the restriction). With F32 coarse fields that start
+ * on 16 bytes, 9 <= nrhs <= 64, 2*ntv a multiple of 8 up to 64 (from 16 on
+ * unless 16 divides nrhs), an engine other than MRHS_DC_ALU and pipeline
+ * stages that fit in shared memory (the split form at 2*ntv = 64 takes up to
+ * 48 right-hand sides) the products run on the tensor cores
  * (tcgen05, FP32 accumulation): split tf32 (hi*hi + hi*lo + lo*hi, FP32
  * accuracy) for FP32 contexts and, in the mixed ones, for nrhs not a multiple
  * of 16; single tf32 for the mixed ones with nrhs a multiple of 16;

@@ -280,9 +280,9 @@ struct Unrecorded {
 // The on-chip smoother's workspace: taken from a pool of the context for one call and
 // given back in stream order, without a synchronisation. Between calls the pool keeps its
 // memory, but as idle pool memory: a cudaMalloc of this process that would run out (of
-// another context, of the caller's own allocator) gets it from the driver. (With what a
-// pool gives back at every synchronisation, or plain allocations, a smoothing of 24 vectors
-// of 32^3 x 64 took 129 ms against 107.)
+// another context, of the caller's own allocator) gets it from the driver. (With a
+// pool that returns its memory at every synchronisation a smoothing of 24 vectors of
+// 32^3 x 64 took 129 ms against 107.)
 struct TileSpace {
   mrhs_ctx c;
   void* p = nullptr;  // nullptr when the memory has run out

@@ -1028,12 +1028,13 @@ static SapGeo sap_face_geo(mrhs_ctx c, int T, size_t* smem) {
 }
 
 // Right-hand sides smoothed together on tile copies: all of them when the workspace (the
-// links and two copies) takes at most tile_limit bytes (20 GB; or 3/4 of what is free), else fewer, so
-// that the largest lattices keep their memory for the setup, in multiples of 8: of a row's
-// 128 bytes (32 right-hand sides) whole 64-byte pieces come from memory, so copies of four
-// at a time cost as much as of eight (48^3 x 96, 32 vectors, a setup: 545 ms in fours,
-// 236 ms in eights, 16 GB). A group is at most kTileGroup, so that k_tiles' rows of one
-// site fit in shared memory. 0: not even four fit, the caller takes the form without copies.
+// links and two copies) takes at most tile_limit bytes (20 GB; or 3/4 of what is free),
+// else fewer, so that the largest lattices keep their memory for the setup, in multiples
+// of 8: of a row's 128 bytes (32 right-hand sides) whole 64-byte pieces come from memory,
+// so copies of four at a time cost as much as of eight (48^3 x 96, 32 vectors, a setup:
+// 545 ms in fours, 236 ms in eights, 16 GB). A group is at most kTileGroup, so that
+// k_tiles' rows of one site fit in shared memory. 0: not even four fit, the caller takes
+// the form without copies.
 constexpr int kTileGroup = 2048;
 static int sap_group(mrhs_ctx c, int nrhs, size_t links) {
   const size_t four = 2 * sizeof(float) * fine_elems(c, 4);
